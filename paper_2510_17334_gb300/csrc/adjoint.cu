@@ -220,104 +220,213 @@ namespace slrf {
 struct MinresScal {
   double beta, oldb, dbar, epsln, phibar, cs, sn, alfa, beta1;
   double oldeps, delta, gamma, phi;
-  int active, iters;
+  int active;   // 1 while the column still iterates
+  int pending;  // 1: the w and x update of the last step is still to come
 };
 
-constexpr int kAdjRows = 512;
+// One MINRES step is two launches: minres_apply_kernel (products with the Lanczos vector, the
+// recurrence's first half, alfa) and minres_update_kernel (its second half, beta, the Givens
+// step and the stopping test).  Blocks of a 32-column tile write partial column sums; the last
+// one adds them in a fixed order and updates the tile's scalars.  The Lanczos vectors rotate
+// through three buffers (no copies), v = r2 / beta is never stored (A v = (A r2) / beta), and
+// the w and x update of a step, which needs only the row's own entries, rides on the next
+// step's apply.  With 11 launches a step and column sums over chunks of 512 rows on one
+// thread each (230 us of latency for 2 x 4 blocks) a step of n = 2,002, k = 16 took 240 us;
+// now 26 us, two launch latencies with their last-block sums (384 steps: 96 -> 9.9 ms).
+constexpr int kAdjWarps = 8;
 
-// partial column sums of x .* y over row chunks: work[chunk][k]
-__global__ void colprod_partial_kernel(int64_t n, int k, const double *x, const double *y, double *work) {
-  const int c = blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  const int64_t r0 = (int64_t)blockIdx.x * kAdjRows;
-  const int64_t r1 = r0 + kAdjRows < n ? r0 + kAdjRows : n;
+// Sum v over the warps of the block and then over the blocks of the tile (gridDim.x of them):
+// true in every thread of the last block, where out is the column's sum in lane c of warp 0.
+__device__ bool tile_reduce(double v, int k, double *part, unsigned *counter, double &out) {
+  __shared__ double sm[kAdjWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.y * 32 + lane;
+  sm[warp][lane] = v;
+  __syncthreads();
+  if (warp == 0 && c < k) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kAdjWarps; ++w) s += sm[w][lane];
+    part[(size_t)blockIdx.x * k + c] = s;
+  }
+  if (!last_block_arrive(counter + blockIdx.y, gridDim.x)) return false;
   double s = 0.0;
-  for (int64_t i = r0; i < r1; ++i) s = fma(x[i * k + c], y[i * k + c], s);
-  work[(size_t)blockIdx.x * k + c] = s;
-}
-static void colprod(int64_t n, int k, const double *x, const double *y, double *work, cudaStream_t st) {
-  dim3 g((unsigned)((n + kAdjRows - 1) / kAdjRows), (k + 127) / 128);
-  colprod_partial_kernel<<<g, 128, 0, st>>>(n, k, x, y, work);
-}
-__device__ __forceinline__ double colprod_final(const double *work, int nch, int k, int c) {
-  double s = 0.0;
-  for (int z = 0; z < nch; ++z) s += work[(size_t)z * k + c];
-  return s;
+  if (c < k) {
+#pragma unroll 8
+    for (unsigned b = warp; b < gridDim.x; b += kAdjWarps) s += __ldcg(part + (size_t)b * k + c);
+  }
+  sm[warp][lane] = s;
+  __syncthreads();
+  out = 0.0;
+#pragma unroll
+  for (int w = 0; w < kAdjWarps; ++w) out += sm[w][lane];
+  if (threadIdx.x == 0) counter[blockIdx.y] = 0u;
+  return true;
 }
 
-// b = -(g - Bx (x^T g)); x^T g from partials
-__global__ void adj_rhs_kernel(int64_t n, int k, const double *g, const double *BX, const double *work, int nch,
-                               double *b) {
+// out[c] = sum over rows of x[:, c] y[:, c]
+__global__ void __launch_bounds__(32 * kAdjWarps) colprod_kernel(int64_t n, int k, int rows, const double *x,
+                                                                 const double *y, double *part, unsigned *counters,
+                                                                 double *out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.y * 32 + lane;
+  const int64_t i0 = (int64_t)blockIdx.x * rows, i1 = i0 + rows < n ? i0 + rows : n;
+  double s = 0.0, tot;
+  if (c < k)
+    for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) s = fma(x[i * k + c], y[i * k + c], s);
+  if (tile_reduce(s, k, part, counters, tot) && warp == 0 && c < k) out[c] = tot;
+}
+
+// b = -(g - Bx (x^T g))
+__global__ void adj_rhs_kernel(int64_t n, int k, const double *g, const double *BX, const double *xg, double *b) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n * k) return;
-  const int c = (int)(t % k);
-  const double xg = colprod_final(work, nch, k, c);
-  b[t] = -(g[t] - BX[t] * xg);
+  b[t] = -(g[t] - BX[t] * xg[t % k]);
 }
 
-// init per column: beta1 = ||b||, r1 = r2 = y = b, x = w = w2 = 0
-__global__ void minres_init_scal_kernel(int k, const double *work, int nch, MinresScal *s) {
+// init per column: beta1 = ||b|| (r2 = b, x = w = w2 = 0)
+__global__ void minres_init_kernel(int k, const double *b2, MinresScal *s) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= k) return;
-  const double b2 = colprod_final(work, nch, k, c);
   MinresScal m{};
-  m.beta1 = sqrt(b2);
+  m.beta1 = sqrt(b2[c]);
   m.beta = m.beta1;
-  m.oldb = 0.0;
-  m.dbar = 0.0;
-  m.epsln = 0.0;
   m.phibar = m.beta1;
   m.cs = -1.0;
-  m.sn = 0.0;
   m.active = m.beta1 > 0.0 ? 1 : 0;
-  m.iters = 0;
   s[c] = m;
 }
 
-// v = y / beta (beta of this step), y = A v - lambda B v - (beta / oldb) r1  [with AV, BV of v]
-__global__ void minres_v_kernel(int64_t n, int k, const double *y, const MinresScal *s, double *v) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * k) return;
-  const int c = (int)(t % k);
-  const MinresScal &m = s[c];
-  v[t] = (m.active && m.beta > 0.0) ? y[t] / m.beta : 0.0;
+struct MinresArgs {
+  int64_t n;
+  int k, rows;  // rows per block
+  const int64_t *rowptr;
+  const int32_t *col;
+  const double *valA, *valB, *lam;
+  const double *r1, *r2;  // Lanczos vectors of the last two steps (unscaled; beta = ||r2||)
+  double *y;              // the next one
+  const double *w;
+  double *w2, *x;
+  MinresScal *s;
+  double *part;
+  unsigned *counters;
+  double tol;
+};
+
+// w and x of the previous step for one entry: w_new = (v - oldeps w2 - delta w) / gamma into w2
+// (the caller swaps the two), x += phi w_new, with v = r1 / oldb that step's Lanczos vector.
+struct MinresW {
+  double iob, oldeps, delta, ig, phi;
+  __device__ explicit MinresW(const MinresScal &m)
+      : iob(1.0 / m.oldb), oldeps(m.oldeps), delta(m.delta), ig(1.0 / m.gamma), phi(m.phi) {}
+  __device__ __forceinline__ void apply(const MinresArgs &a, int64_t t, double r1) const {
+    const double wn = fma(-delta, a.w[t], fma(-oldeps, a.w2[t], r1 * iob)) * ig;
+    a.w2[t] = wn;
+    a.x[t] = fma(phi, wn, a.x[t]);
+  }
+};
+
+// A warp takes a row at a time, cw lanes (8, 16 or 32) over the columns of the tile; with
+// fewer than 32 columns the 32 / cw lane groups share the row's entries.
+template <bool PRODUCT>
+__global__ void __launch_bounds__(32 * kAdjWarps) minres_apply_kernel(const MinresArgs a, int cw) {
+  __shared__ double2 s_ab[kAdjWarps][32];
+  __shared__ int s_c[kAdjWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sub = lane & (cw - 1), part = lane / cw, parts = 32 / cw;
+  const int c = blockIdx.y * 32 + sub;
+  const bool ok = c < a.k;
+  MinresScal m{};
+  if (ok) m = a.s[c];
+  const bool act = PRODUCT && ok && m.active != 0, pend = ok && m.pending != 0;
+  // nothing left to do in this tile (the same for every block: the scalars change only after
+  // all blocks of a launch have arrived)
+  if (!__syncthreads_or(act || pend)) return;
+  const bool own = part == 0;
+  const MinresW wx(m);
+  const double ib = 1.0 / m.beta, ratio = m.oldb > 0.0 ? m.beta / m.oldb : 0.0;
+  const double lam = act ? a.lam[c] : 0.0;
+  const bool any = __any_sync(0xffffffffu, act);
+  const char *const xl = reinterpret_cast<const char *>(a.r2 + (ok ? c : 0));
+  const unsigned row_bytes = (unsigned)a.k * (unsigned)sizeof(double);
+  double sum = 0.0;
+  const int64_t i0 = (int64_t)blockIdx.x * a.rows, i1 = i0 + a.rows < a.n ? i0 + a.rows : a.n;
+  for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) {
+    const int64_t t = i * a.k + c;
+    double sa = 0.0, sb = 0.0, r1 = 0.0, r2 = 0.0;
+    if (own && ok) {
+      if (pend || (act && m.oldb > 0.0)) r1 = a.r1[t];
+      if (act) r2 = a.r2[t];
+    }
+    if (any) {
+      const int64_t rs = a.rowptr[i], re = a.rowptr[i + 1];
+      for (int64_t e0 = rs; e0 < re; e0 += 32) {
+        const int cnt = (int)(re - e0 < 32 ? re - e0 : 32);
+        __syncwarp();
+        if (lane < cnt) {
+          s_c[warp][lane] = a.col[e0 + lane];
+          s_ab[warp][lane] = make_double2(a.valA[e0 + lane], a.valB[e0 + lane]);
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int q = part; q < cnt; q += parts) {
+          const double2 ab = s_ab[warp][q];
+          const double x =
+              *reinterpret_cast<const double *>(xl + (unsigned long long)(unsigned)s_c[warp][q] * row_bytes);
+          sa = fma(ab.x, x, sa);
+          sb = fma(ab.y, x, sb);
+        }
+      }
+      for (int o = cw; o < 32; o <<= 1) {
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+        sb += __shfl_xor_sync(0xffffffffu, sb, o);
+      }
+    }
+    if (own && ok) {
+      if (pend) wx.apply(a, t, r1);
+      if (act) {
+        const double y = fma(-lam, sb, sa) * ib - ratio * r1;
+        a.y[t] = y;
+        sum = fma(r2 * ib, y, sum);
+      }
+    }
+  }
+  double alfa;
+  if (!tile_reduce(sum, a.k, a.part, a.counters, alfa)) return;
+  if (warp == 0 && own && ok) {
+    MinresScal &g = a.s[c];
+    g.alfa = alfa;
+    g.pending = 0;
+  }
 }
-__global__ void minres_apply_kernel(int64_t n, int k, const double *AV, const double *BV, const double *lam,
-                                    const double *r1, const MinresScal *s, double *y) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * k) return;
-  const int c = (int)(t % k);
-  const MinresScal &m = s[c];
-  double val = fma(-lam[c], BV[t], AV[t]);
-  if (m.oldb > 0.0) val -= (m.beta / m.oldb) * r1[t];
-  y[t] = val;
-}
-// alfa = v^T y (final of partials) stored per column
-__global__ void minres_alfa_kernel(int k, const double *work, int nch, MinresScal *s) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  s[c].alfa = colprod_final(work, nch, k, c);
-}
-// y -= (alfa/beta) r2; r1 = r2; r2 = y
-__global__ void minres_y2_kernel(int64_t n, int k, const MinresScal *s, double *y, double *r1, double *r2) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * k) return;
-  const int c = (int)(t % k);
-  const MinresScal &m = s[c];
-  const double yy = m.beta > 0.0 ? y[t] - (m.alfa / m.beta) * r2[t] : y[t];
-  r1[t] = r2[t];
-  r2[t] = yy;
-  y[t] = yy;
-}
-// Givens step with beta_new = ||y|| (final of partials); convergence test
-__global__ void minres_scal_kernel(int k, const double *work, int nch, double tol, int itn, MinresScal *s) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  MinresScal m = s[c];
-  if (!m.active) return;
-  const double bnew = sqrt(colprod_final(work, nch, k, c));
+
+// y -= (alfa / beta) r2; beta_new = ||y||; Givens step; the column stops once
+// phibar <= tol beta1 (its state is frozen after the pending w and x update).
+__global__ void __launch_bounds__(32 * kAdjWarps) minres_update_kernel(const MinresArgs a) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.y * 32 + lane;
+  const bool ok = c < a.k;
+  MinresScal m{};
+  if (ok) m = a.s[c];
+  const bool act = ok && m.active != 0;
+  if (!__syncthreads_or(act)) return;
+  const double ratio = act && m.beta > 0.0 ? m.alfa / m.beta : 0.0;
+  double sum = 0.0;
+  const int64_t i0 = (int64_t)blockIdx.x * a.rows, i1 = i0 + a.rows < a.n ? i0 + a.rows : a.n;
+  if (act) {
+#pragma unroll 4
+    for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) {
+      const int64_t t = i * a.k + c;
+      const double y = a.y[t] - ratio * a.r2[t];
+      a.y[t] = y;
+      sum = fma(y, y, sum);
+    }
+  }
+  double b2;
+  if (!tile_reduce(sum, a.k, a.part, a.counters, b2)) return;
+  if (warp != 0 || !act) return;
   m.oldb = m.beta;
-  m.beta = bnew;
+  m.beta = sqrt(b2);
   m.oldeps = m.epsln;
   m.delta = m.cs * m.dbar + m.sn * m.alfa;
   const double gbar = m.sn * m.dbar - m.cs * m.alfa;
@@ -330,31 +439,9 @@ __global__ void minres_scal_kernel(int k, const double *work, int nch, double to
   m.sn = m.beta / gam;
   m.phi = m.cs * m.phibar;
   m.phibar = m.sn * m.phibar;
-  m.iters = itn;
-  s[c] = m;
-}
-// w1 = w2; w2 = w; w = (v - oldeps w1 - delta w2)/gamma; x += phi w; then the column stops
-// once phibar <= tol beta1 (the state of a stopped column is frozen)
-__global__ void minres_w_kernel(int64_t n, int k, const double *v, const MinresScal *s, double *w, double *w2,
-                                double *x) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * k) return;
-  const int c = (int)(t % k);
-  const MinresScal &m = s[c];
-  if (!m.active) return;
-  const double w1 = w2[t];
-  const double wo = w[t];
-  const double wn = (v[t] - m.oldeps * w1 - m.delta * wo) / m.gamma;
-  w2[t] = wo;
-  w[t] = wn;
-  x[t] = fma(m.phi, wn, x[t]);
-}
-__global__ void minres_stop_kernel(int k, double tol, MinresScal *s, int *notconv, int last) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  MinresScal &m = s[c];
-  if (m.active && (m.phibar <= tol * m.beta1 || m.beta == 0.0)) m.active = 0;
-  if (last && m.active) atomicExch(notconv, 1);
+  m.pending = 1;
+  if (m.phibar <= a.tol * m.beta1 || m.beta == 0.0) m.active = 0;
+  a.s[c] = m;
 }
 __global__ void minres_count_kernel(int k, const MinresScal *s, int *count) {
   int c = 0;
@@ -366,63 +453,79 @@ __global__ void minres_count_kernel(int k, const MinresScal *s, int *count) {
   if (threadIdx.x == 0) *count = sh[0] + sh[1] + sh[2] + sh[3];
 }
 // xi -= x (x^T B xi); then YA = X diag(a) + Xi, YB = X diag(b) + Xi diag(lambda)
-__global__ void adj_finish_kernel(int64_t n, int k, const double *X, const double *xi, const double *work, int nch,
-                                  const double *lam, const double *g_eval, const double *work2, double *YA,
-                                  double *YB) {
+__global__ void adj_finish_kernel(int64_t n, int k, const double *X, const double *xi, const double *xbxi,
+                                  const double *lam, const double *g_eval, const double *gx, double *YA, double *YB) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n * k) return;
   const int c = (int)(t % k);
-  const double xbxi = colprod_final(work, nch, k, c);   // x^T B xi
-  const double gx = colprod_final(work2, nch, k, c);    // g_x^T x
   const double xv = X[t];
-  const double xiv = xi[t] - xv * xbxi;
+  const double xiv = xi[t] - xv * xbxi[c];  // x^T B xi
   YA[t] = g_eval[c] * xv + xiv;
-  YB[t] = (g_eval[c] * lam[c] + 0.5 * gx) * xv + lam[c] * xiv;
+  YB[t] = (g_eval[c] * lam[c] + 0.5 * gx[c]) * xv + lam[c] * xiv;  // g_x^T x
 }
 
 struct AdjBuffers {
-  double *b, *y, *v, *r1, *r2, *w, *w2, *x, *AV, *BV, *YA, *YB, *work, *work2;
+  double *b, *y, *r, *w, *w2, *x, *BV, *YA, *YB;  // n x k blocks
+  double *work, *work2;                           // k words each
   MinresScal *scal;
+  double *part;        // adj_part_doubles(k) words
+  unsigned *counters;  // a zeroed word per 32 columns, left zero
   int *flag;
 };
+
+// Row blocks of the column sums: 16 rows at least, at most 4 blocks a SM and tile.
+static int adj_rows(int64_t n) {
+  const int64_t most = 4 * (int64_t)device_sm_count();
+  const int64_t r = std::max<int64_t>(16, (n + most - 1) / most);
+  return (int)((r + kAdjWarps - 1) / kAdjWarps * kAdjWarps);
+}
+size_t adj_part_doubles(int k) { return 4 * (size_t)device_sm_count() * k; }
+size_t adj_scal_bytes(int k) { return ((size_t)k * sizeof(MinresScal) + 255) / 256 * 256; }
 
 // The caller (slrf.cu) provides n x k scratch blocks (X here has leading dimension k).
 int eig_grad_vectors(int64_t n, const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB,
                      int k, const double *evals, const double *X, const double *g_eval, const double *g_X,
                      double *gA, double *gB, AdjBuffers bf, int maxit, double tol, int *h_active, int *notconv,
                      cudaStream_t st) {
-  const int nch = (int)((n + kAdjRows - 1) / kAdjRows);
   const int64_t tot = n * k;
   const unsigned gb = (unsigned)((tot + 255) / 256);
+  const int rows = adj_rows(n);
+  const dim3 grid((unsigned)((n + rows - 1) / rows), (unsigned)((k + 31) / 32));
+  const int cw = k <= 8 ? 8 : (k <= 16 ? 16 : 32);
+  auto colprod = [&](const double *x, const double *y, double *out) {
+    colprod_kernel<<<grid, 32 * kAdjWarps, 0, st>>>(n, k, rows, x, y, bf.part, bf.counters, out);
+  };
   // right-hand sides
   spmm_real(n, rowptr, col, valA, valB, X, k, k, nullptr, bf.BV, k, st);
-  colprod(n, k, X, g_X, bf.work2, st);  // x^T g
-  adj_rhs_kernel<<<gb, 256, 0, st>>>(n, k, g_X, bf.BV, bf.work2, nch, bf.b);
-  colprod(n, k, bf.b, bf.b, bf.work, st);
-  minres_init_scal_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, bf.work, nch, bf.scal);
-  cudaMemcpyAsync(bf.y, bf.b, tot * sizeof(double), cudaMemcpyDeviceToDevice, st);
-  cudaMemcpyAsync(bf.r1, bf.b, tot * sizeof(double), cudaMemcpyDeviceToDevice, st);
-  cudaMemcpyAsync(bf.r2, bf.b, tot * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  colprod(X, g_X, bf.work2);  // x^T g
+  adj_rhs_kernel<<<gb, 256, 0, st>>>(n, k, g_X, bf.BV, bf.work2, bf.b);
+  colprod(bf.b, bf.b, bf.work);
+  minres_init_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, bf.work, bf.scal);
   cudaMemsetAsync(bf.x, 0, tot * sizeof(double), st);
   cudaMemsetAsync(bf.w, 0, tot * sizeof(double), st);
   cudaMemsetAsync(bf.w2, 0, tot * sizeof(double), st);
-  cudaMemsetAsync(bf.flag, 0, 2 * sizeof(int), st);
+  MinresArgs a{n, k, rows, rowptr, col, valA, valB, evals, bf.r, bf.b, bf.y, bf.w, bf.w2, bf.x, bf.scal, bf.part,
+               bf.counters, tol};
+  // the buffers after a step: r1 = r2, r2 = y, and the w just written in front
+  auto rotate = [&] {
+    double *const w = a.w2;
+    a.w2 = const_cast<double *>(a.w);
+    a.w = w;
+    double *const y = const_cast<double *>(a.r1);
+    a.r1 = a.r2;
+    a.r2 = a.y;
+    a.y = y;
+  };
   *notconv = 0;
+  *h_active = 0;
   int itn = 0;
   while (itn < maxit) {
     const int chunk = maxit - itn < 64 ? maxit - itn : 64;
     for (int j = 0; j < chunk; ++j) {
       ++itn;
-      minres_v_kernel<<<gb, 256, 0, st>>>(n, k, bf.y, bf.scal, bf.v);
-      spmm_real(n, rowptr, col, valA, valB, bf.v, k, k, bf.AV, bf.BV, k, st);
-      minres_apply_kernel<<<gb, 256, 0, st>>>(n, k, bf.AV, bf.BV, evals, bf.r1, bf.scal, bf.y);
-      colprod(n, k, bf.v, bf.y, bf.work, st);
-      minres_alfa_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, bf.work, nch, bf.scal);
-      minres_y2_kernel<<<gb, 256, 0, st>>>(n, k, bf.scal, bf.y, bf.r1, bf.r2);
-      colprod(n, k, bf.y, bf.y, bf.work, st);
-      minres_scal_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, bf.work, nch, tol, itn, bf.scal);
-      minres_w_kernel<<<gb, 256, 0, st>>>(n, k, bf.v, bf.scal, bf.w, bf.w2, bf.x);
-      minres_stop_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, tol, bf.scal, bf.flag, itn == maxit);
+      minres_apply_kernel<true><<<grid, 32 * kAdjWarps, 0, st>>>(a, cw);
+      minres_update_kernel<<<grid, 32 * kAdjWarps, 0, st>>>(a);
+      rotate();
     }
     // how many columns still iterate: stop early when none
     minres_count_kernel<<<1, 128, 0, st>>>(k, bf.scal, bf.flag + 1);
@@ -432,14 +535,13 @@ int eig_grad_vectors(int64_t n, const int64_t *rowptr, const int32_t *col, const
     if (*h_active == 0) break;
   }
   if (maxit > 0 && itn >= maxit && *h_active > 0) *notconv = 1;
+  minres_apply_kernel<false><<<grid, 32 * kAdjWarps, 0, st>>>(a, cw);  // pending w and x updates
   // B-orthogonal projection, then the pattern gradients
   spmm_real(n, rowptr, col, valA, valB, bf.x, k, k, nullptr, bf.BV, k, st);
-  colprod(n, k, X, bf.BV, bf.work, st);  // x^T B xi
-  adj_finish_kernel<<<gb, 256, 0, st>>>(n, k, X, bf.x, bf.work, nch, evals, g_eval, bf.work2, bf.YA, bf.YB);
+  colprod(X, bf.BV, bf.work);  // x^T B xi
+  adj_finish_kernel<<<gb, 256, 0, st>>>(n, k, X, bf.x, bf.work, evals, g_eval, bf.work2, bf.YA, bf.YB);
   // gA[e] = sum_i YA[r][i] X[c][i], gB[e] = -sum_i YB[r][i] X[c][i]
   return sddmm<false>(n, rowptr, col, k, X, k, SdWeights{nullptr, nullptr, bf.YA, bf.YB}, gA, gB, st);
 }
-
-size_t adj_work_doubles(int64_t n, int k) { return (size_t)((n + kAdjRows - 1) / kAdjRows) * k; }
 
 }  // namespace slrf

@@ -28,15 +28,19 @@ int eig_grad_values(int64_t n, const int64_t *rowptr, const int32_t *col, int k,
                     const double *X, int ldx, const double *g, double *gA, double *gB, cudaStream_t st);
 struct MinresScal;
 struct AdjBuffers {
-  double *b, *y, *v, *r1, *r2, *w, *w2, *x, *AV, *BV, *YA, *YB, *work, *work2;
+  double *b, *y, *r, *w, *w2, *x, *BV, *YA, *YB;
+  double *work, *work2;
   MinresScal *scal;
+  double *part;
+  unsigned *counters;
   int *flag;
 };
 int eig_grad_vectors(int64_t n, const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB,
                      int k, const double *evals, const double *X, const double *g_eval, const double *g_X,
                      double *gA, double *gB, AdjBuffers bf, int maxit, double tol, int *h_active, int *notconv,
                      cudaStream_t st);
-size_t adj_work_doubles(int64_t n, int k);
+size_t adj_part_doubles(int k);
+size_t adj_scal_bytes(int k);
 }
 
 struct slrf_ctx {
@@ -1786,10 +1790,15 @@ int slrf_eig_grad(slrf_ctx *ctx, int k, const double *evals, const double *X, in
     copy_block(n, k, X, ldx, ctx->BX, k, ctx->st);
     Xk = ctx->BX;
   }
-  const size_t aw = adj_work_doubles(n, k);
-  if (2 * aw > ctx->work_doubles) return SLRF_EINVAL;
-  AdjBuffers bf{ctx->V, ctx->AV, ctx->BV, ctx->G, ctx->AG, ctx->BG, ctx->U, ctx->U2, ctx->BU, ctx->Vt, ctx->AVt,
-                ctx->BVt, ctx->work, ctx->work + aw, reinterpret_cast<MinresScal *>(ctx->partial), ctx->iflags + 10};
+  // scalars and partial column sums share the COCG partial buffer (4 row blocks per SM of
+  // kNQ doubles per complex column, at least mp of those per real column)
+  unsigned char *const pb = reinterpret_cast<unsigned char *>(ctx->partial);
+  const size_t sb = adj_scal_bytes(k);
+  if (sb + adj_part_doubles(k) * sizeof(double) > (size_t)ctx->sm_count * 4 * ctx->Wmax * kNQ * sizeof(double))
+    return SLRF_EINVAL;
+  AdjBuffers bf{ctx->V, ctx->AV, ctx->G, ctx->BG, ctx->U, ctx->U2, ctx->Vt, ctx->AVt, ctx->BVt, ctx->work,
+                ctx->work + k, reinterpret_cast<MinresScal *>(pb), reinterpret_cast<double *>(pb + sb),
+                ctx->counters, ctx->iflags + 10};
   int notconv = 0;
   const double tol = std::max(ctx->o.tol_inner, 1e-12);
   const int rc = eig_grad_vectors(n, ctx->rowptr, ctx->col, ctx->valA, ctx->valB, k, evals, Xk, g_eval, g_X, gA, gB,

@@ -1,12 +1,15 @@
-"""Eigenvalue adjoint on the pattern (slrf_eig_grad without eigenvector terms) against the sums
-written out in numpy: symmetric patterns (mirrored entries), patterns whose mirror entries are
+"""The adjoint's kernels at the edges of their tiles.  Eigenvalue terms on the pattern against the
+sums written out in numpy: symmetric patterns (mirrored entries), patterns whose mirror entries are
 missing or whose rows are not sorted, even and odd numbers of eigenpairs, row counts around the
 row bundles of a warp."""
 import numpy as np
 import pytest
+import scipy.linalg as sla
 import torch
 
+import slrf_inputs as si
 from gpu_common import slrf_mod  # noqa: F401
+from oracle import slrf_oracle as orc
 
 pytestmark = pytest.mark.gpu
 
@@ -38,4 +41,21 @@ def test_eigenvalue_adjoint_sums(slrf_mod, n, k, form):  # noqa: F811
     bound = (k + 3) * 2.0 ** -53
     assert np.all(np.abs(gA - terms.sum(1)) <= 2 * bound * np.abs(terms).sum(1))
     assert np.all(np.abs(gB + (lam * terms).sum(1)) <= 2 * bound * np.abs(lam * terms).sum(1))
+    ctx.close()
+
+
+@pytest.mark.parametrize("k", [1, 8, 9, 16, 17, 33, 65])
+def test_eigenvector_adjoint_column_tiles(slrf_mod, k):  # noqa: F811
+    """Eigenvector terms at block widths around the lane groups (8, 16, 32 columns) and tiles
+    of the MINRES kernels, against the oracle's dense least squares; the relative residual
+    1e-12 grows by the 1D bar's spread lambda_max / gap < 1e4."""
+    p = si.bar1d_pencil(90)
+    lam, X = sla.eigh(p.A().toarray(), p.B().toarray())
+    lam, X = lam[:k], np.ascontiguousarray(X[:, :k])
+    rng = np.random.default_rng(k)
+    g, gX = rng.standard_normal(k), rng.standard_normal((p.n, k))
+    ctx = slrf_mod.Context(p.rowptr, p.col, p.valA, p.valB, 1.0, k, slrf_mod.slrf_opts_default(tol_inner=1e-13))
+    out = ctx.eig_grad(*(torch.from_numpy(t) for t in (lam, X, g, gX)))
+    for got, want in zip(out, orc.eig_grad_full(p.rowptr, p.col, p.A(), p.B(), lam, X, g, gX)):
+        assert np.abs(got.cpu().numpy() - want).max() <= 1e-8 * np.abs(want).max()
     ctx.close()
