@@ -164,25 +164,31 @@ __device__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], const int W, cons
     partial[((size_t)rb * W + w_tile0 + wl) * kNQ + qq] = s;
   }
   if (!last_block_arrive(counter, (unsigned)nrb)) return false;
-  // last block: sum the nrb slots of this tile in a fixed order
-  double a2[VEC][NQ];
-#pragma unroll
-  for (int v = 0; v < VEC; ++v)
-#pragma unroll
-    for (int qq = 0; qq < NQ; ++qq) a2[v][qq] = 0.0;
-  for (int b = warp; b < nrb; b += kWarps) {
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) {
-      const double *src = partial + ((size_t)b * W + w_tile0 + lane * VEC + v) * kNQ;
-#pragma unroll
-      for (int qq = 0; qq < NQ; ++qq) a2[v][qq] += __ldcg(src + qq);
-    }
-  }
+  // last block: sum the nrb slots of this tile in a fixed order, a thread per value (or per
+  // value and slice of the slots, where there are fewer values than threads).  The sums sit on
+  // the critical path of every launch, so each thread keeps 8 loads in flight; a slot at a time
+  // (all values of a column per thread) they took nrb / 8 L2 round trips.
+  constexpr int NV = TW * NQ;
+  constexpr int SL = NV < kThreads ? kThreads / NV : 1;
+  static_assert(SL * NV <= kWarps * NV, "slices fit the shared array");
+  double *const sums = &sm[0][0][0];
   __syncthreads();
+  for (int t = threadIdx.x; t < NV * SL; t += kThreads) {
+    const int val = t % NV, slice = t / NV;
+    const double *src = partial + ((size_t)w_tile0 + val / NQ) * kNQ + val % NQ;
+    const size_t step = (size_t)W * kNQ;
+    double s = 0.0;
+    int b = slice;
+    for (; b + 7 * SL < nrb; b += 8 * SL) {
+      double x[8];
 #pragma unroll
-  for (int v = 0; v < VEC; ++v)
+      for (int u = 0; u < 8; ++u) x[u] = __ldcg(src + (size_t)(b + u * SL) * step);
 #pragma unroll
-    for (int qq = 0; qq < NQ; ++qq) sm[warp][lane * VEC + v][qq] = a2[v][qq];
+      for (int u = 0; u < 8; ++u) s += x[u];
+    }
+    for (; b < nrb; b += SL) s += __ldcg(src + (size_t)b * step);
+    sums[t] = s;
+  }
   __syncthreads();
   if (threadIdx.x < TW) {
     w_out = w_tile0 + threadIdx.x;
@@ -190,7 +196,7 @@ __device__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], const int W, cons
     for (int qq = 0; qq < NQ; ++qq) {
       double s = 0.0;
 #pragma unroll
-      for (int wi = 0; wi < kWarps; ++wi) s += sm[wi][threadIdx.x][qq];
+      for (int i = 0; i < SL; ++i) s += sums[i * NV + threadIdx.x * NQ + qq];
       out[qq] = s;
     }
   }
