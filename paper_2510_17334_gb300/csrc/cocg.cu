@@ -240,10 +240,34 @@ __device__ __forceinline__ void cocg_init_body(const CocgArgs<R> &a, const int r
   const int64_t i1 = (i0 + a.rows_per_block < a.n ? i0 + a.rows_per_block : a.n);
   for (int64_t i = i0 + warp; i < i1; i += kWarps) {
     Vec<R, VEC> rv, qv;
+    // FP32: g, A g and B g of a column are converted once, by different lanes of the column,
+    // and shared by shuffles.  GB300 converts FP64 on its FP64 pipe (2 per clock and SM); with
+    // every lane converting for each of its poles the conversions alone took 0.46 ms at
+    // n W = 88M (41^3 nodes, 160 columns, 8 poles): 0.84 -> 0.63 ms.
+    R gsh[3] = {R(0), R(0), R(0)};
+    const bool shared_col = sizeof(R) == 4 && a.mp >= VEC;
+    if (shared_col) {
+      const int lpc = a.mp / VEC, sub = lane & (lpc - 1);
+      R own[3] = {R(0), R(0), R(0)};
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int q = t * lpc + sub;  // 0: g, 1: A g, 2: B g
+        if (q < 3 && ok[0]) {
+          const double *src = q == 0 ? a.g : (q == 1 ? a.Ag : a.Bg);
+          const size_t o = (size_t)i * a.ldg + cidx[0];
+          if (CHK(1, o, (long long)a.n * a.ldg)) own[t] = (R)src[o];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const R x = q < lpc ? own[0] : (lpc == 2 ? own[1] : own[q]);  // slot q / lpc
+        gsh[q] = __shfl_sync(0xffffffffu, x, (lane - sub) + (q & (lpc - 1)));
+      }
+    }
 #pragma unroll
     for (int v = 0; v < VEC; ++v) {
-      R gv = 0, agv = 0, bgv = 0;
-      if (ok[v]) {
+      R gv = gsh[0], agv = gsh[1], bgv = gsh[2];
+      if (!shared_col && ok[v]) {
         const size_t o = (size_t)i * a.ldg + cidx[v];
         if (CHK(1, o, (long long)a.n * a.ldg)) { gv = (R)a.g[o]; agv = (R)a.Ag[o]; bgv = (R)a.Bg[o]; }
       }
