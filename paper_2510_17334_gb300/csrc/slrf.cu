@@ -404,11 +404,10 @@ struct FilterTiming {
   int n_spmm = 0, n_update = 0;
 };
 
-// Row blocks per column tile before autotuning.  Plain CSR: about as many as the GPU
-// holds resident (SMs x 4 blocks), so that the blocks in flight at any time all belong to
-// one or two tiles (the tile index varies slowest) and the gathered rows of those tiles stay
-// in L2.  Grouped SpMM: exactly one resident wave of that kernel, whose blocks take
-// interleaved stripes of groups and so sweep the rows of a tile together.
+// Most row blocks per column tile before autotuning.  Plain CSR: as many as the GPU holds
+// resident (SMs x 4 blocks); csr_rows chooses fewer.  Grouped SpMM: exactly one resident wave of
+// that kernel, whose blocks take interleaved stripes of groups and so sweep the rows of a tile
+// together.
 static int64_t row_blocks(const slrf_ctx *ctx) {
   const int per_sm = (ctx->grp > 1 && ctx->grp_bpsm > 0) ? std::min(ctx->grp_bpsm, 4) : 4;
   return (int64_t)ctx->sm_count * per_sm;
@@ -440,16 +439,47 @@ static void real_products64(slrf_ctx *ctx, const double *X, int ldx, int k, doub
     spmm_real(ctx->n, ctx->rowptr, ctx->col, ctx->valA, ctx->valB, X, ldx, k, YA, YB, ldy, st);
 }
 
+// Rows per block of the plain-CSR COCG launches.  A block costs a fixed latency (start, block
+// reduction, arrival at the tile's counter) and its rows' share of the SM, and a tile's last
+// block sums one slot per row block; for small problems the split that fills the row_blocks()
+// limit (16 rows a block) is mostly that latency.  The model, in microseconds, is fitted to
+// timings of GB300 between n = 930 and 68,921: a block 6 + 0.13 a row, four at a time on an SM;
+// the SM's throughput 0.02 + 0.0036 per stored entry and row in FP32, 0.1 + 0.035 in FP64 (its
+// FP64 pipe); 0.05 per row block in the last block's sum.  At most 128 rows, so that the
+// gathered rows of the blocks in flight (4 an SM, 512 bytes a row) stay within a third of L2.
+// `row_tiles`: rows x column tiles of the launch (over all problems of an FP32 batch).
+// FP32, It_max 8, 20^3 nodes, 32 columns: 16 rows a block 1.46 ms, 48 rows 0.89 ms; a solve of
+// 21 x 20 x 19 nodes, block 100: 182 -> 136 ms; 41^3 nodes, 160 columns: 120 rows 18.3 ms,
+// 128 rows 18.0 ms, 256 rows 20.1 ms.
+static int64_t csr_rows(const slrf_ctx *ctx, double row_tiles, bool fp32) {
+  const int64_t sms = ctx->sm_count, n = ctx->n;
+  const double nnz_row = (double)ctx->nnz / n, tiles = std::max(1.0, row_tiles / n);
+  const double thr = fp32 ? 0.02 + 0.0036 * nnz_row : 0.1 + 0.035 * nnz_row;
+  const int64_t least = (n + 4 * sms - 1) / (4 * sms);  // the partial sums hold 4 row blocks per SM
+  int64_t best = (least + kWarps - 1) / kWarps * kWarps;
+  double best_cost = 1e300;
+  for (int64_t r = best; r <= std::max<int64_t>(best, 128); r += kWarps) {
+    const double nrb = (double)((n + r - 1) / r), blocks = std::ceil(nrb * tiles);
+    const double cost = std::ceil(blocks / sms) * r * thr + std::ceil(blocks / (4 * sms)) * (6.0 + 0.13 * r) + 0.05 * nrb;
+    if (cost < best_cost) { best_cost = cost; best = r; }
+  }
+  return best;
+}
+
 // COCG arguments of one filter apply of this context (k columns, optional warm start).
 template <typename R>
-static CocgArgs<R> build_cocg_args(slrf_ctx *ctx, const double *X, int ldx, int k, double *U, int ldu, int &nref) {
+static CocgArgs<R> build_cocg_args(slrf_ctx *ctx, const double *X, int ldx, int k, double *U, int ldu, int &nref,
+                                   double row_tiles = 0.0) {
   const int vec = ctx->vec;  // lane width of the SpMM format in use
   const int kp = kpad_of(k, ctx->mp, vec);
   const int W = kp * ctx->mp;
-  // row blocks per tile (row_blocks); an autotuned row count (slrf_opts.autotune) replaces it
+  // rows per block (csr_rows; grouped SpMM: row_blocks); an autotuned count (slrf_opts.autotune)
+  // replaces it
   const int64_t rblocks = row_blocks(ctx);
   int64_t rpb = std::max<int64_t>(16, (ctx->n + rblocks - 1) / rblocks);
   if (ctx->rpb_tuned > 0) rpb = std::max<int64_t>(rpb, ctx->rpb_tuned);
+  else if (ctx->grp == 1)
+    rpb = csr_rows(ctx, row_tiles > 0.0 ? row_tiles : (double)ctx->n * (W / (32 * vec)), sizeof(R) == 4);
   // whole groups per row block, the same number for every warp of the block
   const int64_t unit = (int64_t)ctx->grp * kWarps;
   rpb = (rpb + unit - 1) / unit * unit;
@@ -908,13 +938,18 @@ static int batch_outer_filter(slrf_batch *b, const std::vector<int> &act, const 
   int nref = 1, total = 0, itm = 0;
   const int P = (int)act.size();
   b->hprefix[0] = 0;
+  // FP32: the rows per block follow the whole launch; FP64 keeps each problem's own, so that a
+  // batch stays bitwise equal to single solves
+  double row_tiles = 0.0;
+  if (sizeof(R) == 4)
+    for (int p : act) row_tiles += (double)b->c[p]->n * (kpad_of(kk[p], b->c[p]->mp, vec) * b->c[p]->mp / (32 * vec));
   for (int i = 0; i < P; ++i) {
     slrf_ctx *c = b->c[act[i]];
     const int k = kk[act[i]];
     const double *th = warm[act[i]] ? c->theta_act : nullptr;
     int rc = filter_prep(c, c->V, c->L, k, th, warm[act[i]] ? c->AV : nullptr, warm[act[i]] ? c->BV : nullptr);
     if (rc != SLRF_OK) return rc;
-    ha[i] = build_cocg_args<R>(c, c->V, c->L, k, c->U, c->L, nref);
+    ha[i] = build_cocg_args<R>(c, c->V, c->L, k, c->U, c->L, nref, row_tiles);
     ha[i].it_cap = c->o.it_adapt ? c->it_cur : 0;  // per-problem It_max inside the shared loop
     if (ha[i].vec != vec || ha[i].G != 1) return SLRF_EINVAL;  // the batched setup forces group = 1
     for (int step = 1; step <= nref; ++step) {  // the batched kernels read these buffers unchecked
