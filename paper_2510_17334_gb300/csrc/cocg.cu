@@ -23,6 +23,7 @@
 // them in a fixed order (deterministic) and updates the per-column scalars.
 #include "cocg.cuh"
 
+#include <algorithm>
 #include <type_traits>
 
 #ifndef SLRF_GATHER_UNROLL
@@ -63,19 +64,19 @@ namespace slrf {
 // VEC complex entries of one lane (16-byte loads: one in FP64, VEC / 2 in FP32)
 template <typename R, int V> struct Vec { cx_t<R> z[V]; };
 
-// Where the lane's 16-byte pieces live.  The kernels index the complex state (r, p, q, d)
-// logically -- lane l owns the entries [V l, V l + V) of a tile of 32 V -- and reach it only
-// through ldv / stv at tile + V l.  With V > 2 (FP32, two pieces per lane) the pieces are
-// stored 64 entries apart, piece j of lane l at tile + 64 j + 2 l, so that every load
-// instruction of the warp covers 512 contiguous bytes (with the pieces side by side, each
-// instruction would touch every sector of the 1 KB segment and use half of it).
+// Which entries of a tile of 32 V a lane owns.  The state is linear in w; a lane's 16-byte
+// pieces (one complex in FP64, two in FP32) sit 64 entries apart where it has several (V = 4),
+// so that every load instruction of the warp covers 512 contiguous bytes (with the pieces side
+// by side, each instruction would touch every sector of the 1 KB segment and use half of it).
+// Lane base lane_w, entry v at lane_w + woff(v); piece_len entries of a piece are adjacent.
+template <int V> __host__ __device__ constexpr int piece_len() { return V > 2 ? 2 : V; }
+template <int V> __host__ __device__ constexpr int woff(int v) { return V > 2 ? 64 * (v / 2) + v % 2 : v; }
+template <int V> __device__ __forceinline__ int lane_w(int lane) { return lane * piece_len<V>(); }
 template <typename R, int V> __device__ __forceinline__ const float4 *piece(const cx_t<R> *p, int j) {
-  const int lane = threadIdx.x & 31;
-  return reinterpret_cast<const float4 *>(p - (V - 2) * lane + 64 * j);
+  return reinterpret_cast<const float4 *>(p + 64 * j);
 }
 template <typename R, int V> __device__ __forceinline__ float4 *piece(cx_t<R> *p, int j) {
-  const int lane = threadIdx.x & 31;
-  return reinterpret_cast<float4 *>(p - (V - 2) * lane + 64 * j);
+  return reinterpret_cast<float4 *>(p + 64 * j);
 }
 
 template <typename R, int V> __device__ __forceinline__ Vec<R, V> ldv(const cx_t<R> *p) {
@@ -147,14 +148,14 @@ template <typename R> __device__ __forceinline__ cx_t<R> to_c(double2 a) {
 template <int VEC, int NQ>
 __device__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], const int W, const int w_tile0,
                                        const int rb, const int nrb, double *partial,
-                                       unsigned *counter, double (&out)[NQ], int &w_out) {
+                                       unsigned *counter, double (&out)[NQ], int &w_out,
+                                       double (*sm)[32 * VEC][NQ]) {
   constexpr int TW = 32 * VEC;
-  __shared__ double sm[kWarps][TW][NQ];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int v = 0; v < VEC; ++v)
 #pragma unroll
-    for (int qq = 0; qq < NQ; ++qq) sm[warp][lane * VEC + v][qq] = acc[v][qq];
+    for (int qq = 0; qq < NQ; ++qq) sm[warp][lane_w<VEC>(lane) + woff<VEC>(v)][qq] = acc[v][qq];
   __syncthreads();
   for (int t = threadIdx.x; t < TW * NQ; t += kThreads) {
     const int wl = t / NQ, qq = t % NQ;
@@ -204,6 +205,15 @@ __device__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], const int W, cons
   return true;
 }
 
+// The same with its scratch ([kWarps][32 VEC][NQ] doubles) in static shared memory.
+template <int VEC, int NQ>
+__device__ __forceinline__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], const int W, const int w_tile0,
+                                                       const int rb, const int nrb, double *partial,
+                                                       unsigned *counter, double (&out)[NQ], int &w_out) {
+  __shared__ double sm[kWarps][32 * VEC][NQ];
+  return block_then_grid_reduce<VEC, NQ>(acc, W, w_tile0, rb, nrb, partial, counter, out, w_out, sm);
+}
+
 // ------------------------------------------------------------------------------ init
 // r0 = c g, p0 = r0, q0 = c (A g - sigma B g); reduce mu0 = p0^T q0, rho0 = r0^T r0, ||r0||^2.
 template <typename R, int V>
@@ -212,13 +222,13 @@ __device__ __forceinline__ void cocg_init_body(const CocgArgs<R> &a, const int r
   using C = cx_t<R>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
-  const int w0 = w_tile0 + lane * VEC;
+  const int w0 = w_tile0 + lane_w<V>(lane);
   C sg[VEC], cf[VEC];
   int cidx[VEC];
   bool ok[VEC];
 #pragma unroll
   for (int v = 0; v < VEC; ++v) {
-    const int w = w0 + v;
+    const int w = w0 + woff<V>(v);
     sg[v] = a.sig[w & (a.mp - 1)];
     cidx[v] = w / a.mp;
     ok[v] = cidx[v] < a.k;
@@ -244,30 +254,36 @@ __device__ __forceinline__ void cocg_init_body(const CocgArgs<R> &a, const int r
     // and shared by shuffles.  GB300 converts FP64 on its FP64 pipe (2 per clock and SM); with
     // every lane converting for each of its poles the conversions alone took 0.46 ms at
     // n W = 88M (41^3 nodes, 160 columns, 8 poles): 0.84 -> 0.63 ms.
-    R gsh[3] = {R(0), R(0), R(0)};
-    const bool shared_col = sizeof(R) == 4 && a.mp >= VEC;
+    constexpr int PL = piece_len<V>(), NP = VEC / PL;
+    R gsh[NP][3];
+    const bool shared_col = sizeof(R) == 4 && a.mp >= PL;
     if (shared_col) {
-      const int lpc = a.mp / VEC, sub = lane & (lpc - 1);
-      R own[3] = {R(0), R(0), R(0)};
+      const int lpc = a.mp / PL, sub = lane & (lpc - 1);
 #pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        const int q = t * lpc + sub;  // 0: g, 1: A g, 2: B g
-        if (q < 3 && ok[0]) {
-          const double *src = q == 0 ? a.g : (q == 1 ? a.Ag : a.Bg);
-          const size_t o = (size_t)i * a.ldg + cidx[0];
-          if (CHK(1, o, (long long)a.n * a.ldg)) own[t] = (R)src[o];
+      for (int j = 0; j < NP; ++j) {
+        R own[3] = {R(0), R(0), R(0)};
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const int q = t * lpc + sub;  // 0: g, 1: A g, 2: B g
+          if (q < 3 && ok[j * PL]) {
+            const double *src = q == 0 ? a.g : (q == 1 ? a.Ag : a.Bg);
+            const size_t o = (size_t)i * a.ldg + cidx[j * PL];
+            if (CHK(1, o, (long long)a.n * a.ldg)) own[t] = (R)src[o];
+          }
         }
-      }
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const R x = q < lpc ? own[0] : (lpc == 2 ? own[1] : own[q]);  // slot q / lpc
-        gsh[q] = __shfl_sync(0xffffffffu, x, (lane - sub) + (q & (lpc - 1)));
+        for (int q = 0; q < 3; ++q) {
+          const R x = q < lpc ? own[0] : (lpc == 2 ? own[1] : own[q]);  // slot q / lpc
+          gsh[j][q] = __shfl_sync(0xffffffffu, x, (lane - sub) + (q & (lpc - 1)));
+        }
       }
     }
 #pragma unroll
     for (int v = 0; v < VEC; ++v) {
-      R gv = gsh[0], agv = gsh[1], bgv = gsh[2];
-      if (!shared_col && ok[v]) {
+      R gv = 0, agv = 0, bgv = 0;
+      if (shared_col) {
+        gv = gsh[v / PL][0]; agv = gsh[v / PL][1]; bgv = gsh[v / PL][2];
+      } else if (ok[v]) {
         const size_t o = (size_t)i * a.ldg + cidx[v];
         if (CHK(1, o, (long long)a.n * a.ldg)) { gv = (R)a.g[o]; agv = (R)a.Ag[o]; bgv = (R)a.Bg[o]; }
       }
@@ -282,7 +298,7 @@ __device__ __forceinline__ void cocg_init_body(const CocgArgs<R> &a, const int r
       acc[v][4] += r0.x * r0.x + r0.y * r0.y;
     }
     const size_t off = (size_t)i * a.W + w0;
-    if (CHK(2, off + VEC - 1, (long long)a.n * a.W)) {
+    if (CHK(2, off + woff<V>(VEC - 1), (long long)a.n * a.W)) {
       stv<R, VEC>(a.r + off, rv);
       stv<R, VEC>(a.p + off, rv);
       stv<R, VEC>(a.q + off, qv);
@@ -333,18 +349,21 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
   using C = cx_t<R>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
-  const int w0 = w_tile0 + lane * VEC;
+  const int w0 = w_tile0 + lane_w<V>(lane);
   C al[VEC];
-  double2 wt[VEC];  // weights stay FP64: the pole sum is formed in FP64
+  constexpr int PL = piece_len<V>();  // entries of a piece share a column when mp >= PL
+  // weights stay FP64: the pole sum is formed in FP64 (the pieces, 64 entries apart, have the
+  // same poles: mp divides 32)
+  double2 wt[PL];
   bool act[VEC];
   bool any_act = false;
 #pragma unroll
   for (int v = 0; v < VEC; ++v) {
-    const WScal &s = a.ws[w0 + v];
+    const WScal &s = a.ws[w0 + woff<V>(v)];
     act[v] = s.active != 0;
     any_act |= act[v];
     al[v] = to_c<R>(s.alpha);
-    wt[v] = a.wt[(w0 + v) & (a.mp - 1)];
+    if (v < PL) wt[v] = a.wt[(w0 + v) & (a.mp - 1)];
   }
   constexpr int NQ = 3;
   R acc[VEC][NQ];  // per-thread partial sums in the working precision
@@ -354,7 +373,7 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
     for (int qq = 0; qq < NQ; ++qq) acc[v][qq] = R(0);
   const int64_t i0 = (int64_t)rb * a.rows_per_block;
   const int64_t i1 = (i0 + a.rows_per_block < a.n ? i0 + a.rows_per_block : a.n);
-  const int lanes_per_col = a.mp >= VEC ? a.mp / VEC : 1;
+  const int lanes_per_col = a.mp >= PL ? a.mp / PL : 1;
   const bool warp_act = __any_sync(0xffffffffu, any_act);
   const int cpt = 32 * VEC / a.mp;  // columns of a tile (kAccU accumulator layout)
 #pragma unroll 1
@@ -372,8 +391,8 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
         uold[v] = R(0);
-        const int c = (w0 + v) / a.mp;
-        const bool lead = a.mp >= VEC ? (v == 0 && (lane % lanes_per_col) == 0) : true;
+        const int c = (w0 + woff<V>(v)) / a.mp;
+        const bool lead = a.mp >= PL ? (v % PL == 0 && (lane % lanes_per_col) == 0) : true;
         if (!FIRST && (warp_act || ACCU_END) && lead && c < a.k) uold[v] = uacc[c];
       }
     } else {
@@ -381,12 +400,12 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
 #pragma unroll
         for (int v = 0; v < VEC; ++v) dv.z[v] = cmake<C>(0, 0);
       } else if (any_act || FINAL) {
-        if (CHK(3, off + VEC - 1, (long long)a.n * a.W)) dv = ldv<R, VEC>(a.d + off);
+        if (CHK(3, off + woff<V>(VEC - 1), (long long)a.n * a.W)) dv = ldv<R, VEC>(a.d + off);
       }
     }
     if (any_act) {
       Vec<R, VEC> pv, qv, rv;
-      if (CHK(4, off + VEC - 1, (long long)a.n * a.W)) {
+      if (CHK(4, off + woff<V>(VEC - 1), (long long)a.n * a.W)) {
         pv = ldv<R, VEC>(a.p + off);
         qv = ldv<R, VEC>(a.q + off);
         rv = ldv<R, VEC>(a.r + off);
@@ -396,7 +415,7 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
         if (act[v]) {
           if constexpr (ACCU) {
             const C ap = cmul(al[v], pv.z[v]);
-            step[v] = R(2) * ((R)wt[v].x * ap.x - (R)wt[v].y * ap.y);
+            step[v] = R(2) * ((R)wt[v % PL].x * ap.x - (R)wt[v % PL].y * ap.y);
           } else {
             dv.z[v] = cfma(al[v], pv.z[v], dv.z[v]);
           }
@@ -407,7 +426,7 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
         acc[v][1] += 2 * rr.x * rr.y;
         acc[v][2] += rr.x * rr.x + rr.y * rr.y;
       }
-      if (CHK(5, off + VEC - 1, (long long)a.n * a.W)) stv<R, VEC>(a.r + off, rv);
+      if (CHK(5, off + woff<V>(VEC - 1), (long long)a.n * a.W)) stv<R, VEC>(a.r + off, rv);
     }
     if constexpr (ACCU) {
       if (FIRST || ACCU_END || warp_act) {
@@ -422,32 +441,35 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
             uacc[c] = acc_new;
           }
         };
-        if (a.mp >= VEC) {
-          R sum = R(0);
+        if (a.mp >= PL) {
 #pragma unroll
-          for (int v = 0; v < VEC; ++v) sum += step[v];
-          for (int o = lanes_per_col >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          const int c = w0 / a.mp;
-          if ((lane % lanes_per_col) == 0 && c < a.k) put(c, uold[0] + sum);
+          for (int j = 0; j < VEC / PL; ++j) {
+            R sum = R(0);
+#pragma unroll
+            for (int v = 0; v < PL; ++v) sum += step[j * PL + v];
+            for (int o = lanes_per_col >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            const int c = (w0 + woff<V>(j * PL)) / a.mp;
+            if ((lane % lanes_per_col) == 0 && c < a.k) put(c, uold[j * PL] + sum);
+          }
         } else {
 #pragma unroll
           for (int v = 0; v < VEC; ++v) {
-            const int c = (w0 + v) / a.mp;
+            const int c = (w0 + woff<V>(v)) / a.mp;
             if (c < a.k) put(c, uold[v] + step[v]);
           }
         }
       }
       continue;
     }
-    if ((FIRST || any_act) && CHK(6, off + VEC - 1, (long long)a.n * a.W)) stv<R, VEC>(a.d + off, dv);
+    if ((FIRST || any_act) && CHK(6, off + woff<V>(VEC - 1), (long long)a.n * a.W)) stv<R, VEC>(a.d + off, dv);
     if (FM == kFinalStoreD || FM == kFinalAddD) {
       // refinement: accumulate this step's correction into the FP64 D
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
-        double2 acc2 = FM == kFinalAddD ? a.D64[off + v] : make_double2(0.0, 0.0);
+        double2 acc2 = FM == kFinalAddD ? a.D64[off + woff<V>(v)] : make_double2(0.0, 0.0);
         acc2.x += (double)dv.z[v].x;
         acc2.y += (double)dv.z[v].y;
-        a.D64[off + v] = acc2;
+        a.D64[off + woff<V>(v)] = acc2;
       }
     } else if (FINAL) {
       // U = coefV V + sum over this column's poles of 2 Re(w_j y_j), y_j = d_j (+ D_j)
@@ -456,30 +478,33 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
       for (int v = 0; v < VEC; ++v) {
         double yr = (double)dv.z[v].x, yi = (double)dv.z[v].y;
         if (FM == kFinalUFromD) {
-          const double2 dd = a.D64[off + v];
+          const double2 dd = a.D64[off + woff<V>(v)];
           yr += dd.x;
           yi += dd.y;
         }
-        part[v] = 2.0 * (wt[v].x * yr - wt[v].y * yi);
+        part[v] = 2.0 * (wt[v % PL].x * yr - wt[v % PL].y * yi);
       }
       // preconditioned solves work on z = D^1/2 y: y = dsc_i z
       const double ds = a.dsc != nullptr ? a.dsc[i] : 1.0;
-      if (a.mp >= VEC) {
-        double s = 0.0;
+      if (a.mp >= PL) {
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) s += part[v];
-        for (int o = lanes_per_col >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const int c = w0 / a.mp;
-        if ((lane % lanes_per_col) == 0 && c < a.k) {
-          if (a.gscale != nullptr) s /= a.gscale[c];
-          if (a.dsc != nullptr) s *= ds;
-          if (CHK(7, (long long)i * a.ldu + c, (long long)a.n * a.ldu) && CHK(8, c, a.k))
-            a.U[(size_t)i * a.ldu + c] = a.coefV[c] * a.V[(size_t)i * a.ldv + c] + s;
+        for (int j = 0; j < VEC / PL; ++j) {
+          double s = 0.0;
+#pragma unroll
+          for (int v = 0; v < PL; ++v) s += part[j * PL + v];
+          for (int o = lanes_per_col >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          const int c = (w0 + woff<V>(j * PL)) / a.mp;
+          if ((lane % lanes_per_col) == 0 && c < a.k) {
+            if (a.gscale != nullptr) s /= a.gscale[c];
+            if (a.dsc != nullptr) s *= ds;
+            if (CHK(7, (long long)i * a.ldu + c, (long long)a.n * a.ldu) && CHK(8, c, a.k))
+              a.U[(size_t)i * a.ldu + c] = a.coefV[c] * a.V[(size_t)i * a.ldv + c] + s;
+          }
         }
       } else {
 #pragma unroll
         for (int v = 0; v < VEC; ++v) {
-          const int c = (w0 + v) / a.mp;
+          const int c = (w0 + woff<V>(v)) / a.mp;
           if (c < a.k) {
             double s = a.gscale ? part[v] / a.gscale[c] : part[v];
             if (a.dsc != nullptr) s *= ds;
@@ -551,9 +576,11 @@ template <> __device__ __forceinline__ void srec_get<double>(const SRec<double> 
 
 // Block and grid reduction of the mu partials of one SpMM launch, then alpha = rho / mu per
 // (pole, column) in the last block of the tile (breakdown: mu = 0 or not finite).
-template <typename R, int VEC>
+// SHARED: the reduction's scratch is the caller's (scratch), else static shared memory.
+template <typename R, int VEC, bool SHARED = false>
 __device__ __forceinline__ void spmm_tail(const CocgArgs<R> &a, const R (&acc)[VEC][2], const int w_tile0,
-                                          const int rb, const int tile, const int nblocks) {
+                                          const int rb, const int tile, const int nblocks,
+                                          double *scratch = nullptr) {
   constexpr int NQ = 2;
   double out[NQ];
   int w;
@@ -562,8 +589,13 @@ __device__ __forceinline__ void spmm_tail(const CocgArgs<R> &a, const R (&acc)[V
   for (int v = 0; v < VEC; ++v)
 #pragma unroll
     for (int qq = 0; qq < NQ; ++qq) accd[v][qq] = (double)acc[v][qq];
-  if (!block_then_grid_reduce<VEC, NQ>(accd, a.W, w_tile0, rb, nblocks, a.partial, a.counters + tile, out, w))
-    return;
+  bool last;
+  if constexpr (SHARED)
+    last = block_then_grid_reduce<VEC, NQ>(accd, a.W, w_tile0, rb, nblocks, a.partial, a.counters + tile, out, w,
+                                           reinterpret_cast<double (*)[32 * VEC][NQ]>(scratch));
+  else
+    last = block_then_grid_reduce<VEC, NQ>(accd, a.W, w_tile0, rb, nblocks, a.partial, a.counters + tile, out, w);
+  if (!last) return;
   if (threadIdx.x < 32 * VEC) {
     WScal s = a.ws[w];
     if (s.active) {
@@ -587,14 +619,14 @@ __device__ __forceinline__ void cocg_spmm_body(const CocgArgs<R> &a, const int r
   using C = cx_t<R>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
-  const int w0 = w_tile0 + lane * VEC;
+  const int w0 = w_tile0 + lane_w<V>(lane);
   constexpr bool kSrec = sizeof(R) == 8 ? SLRF_SPMM_SREC64 != 0 : SLRF_SPMM_SREC32 != 0;
   __shared__ SRec<R> srec_all[kSrec ? kWarps * 32 : 1];
   SRec<R> *const srec = srec_all + (kSrec ? warp * 32 : 0);
   // (beta and the poles are read again for each row's epilogue: not held across the gathers)
   bool any_act = false;
 #pragma unroll
-  for (int v = 0; v < VEC; ++v) any_act |= a.ws[w0 + v].active != 0;
+  for (int v = 0; v < VEC; ++v) any_act |= a.ws[w0 + woff<V>(v)].active != 0;
   // warp-uniform: skip the tile's SpMM when no column in it is still iterating
   const bool warp_act = __any_sync(0xffffffffu, any_act);
   constexpr int NQ = 2;
@@ -654,8 +686,8 @@ __device__ __forceinline__ void cocg_spmm_body(const CocgArgs<R> &a, const int r
       const size_t off = (size_t)i * a.W + w0;
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
-        const C be = to_c<R>(a.ws[w0 + v].beta);
-        const C sg = a.sig[(w0 + v) & (a.mp - 1)];
+        const C be = to_c<R>(a.ws[w0 + woff<V>(v)].beta);
+        const C sg = a.sig[(w0 + woff<V>(v)) & (a.mp - 1)];
         const C s = cfms(sg, sb[v], sa[v]);  // A r - sigma B r
         // a fresh start (refinement step) has p = r and q = (A - sigma B) r
         const C pn = FRESH ? rv.z[v] : cfma(be, pv.z[v], rv.z[v]);
@@ -899,11 +931,11 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
-  const int w0 = w_tile0 + lane * VEC;
+  const int w0 = w_tile0 + lane_w<V>(lane);
   // (beta and the poles are read again in each group's epilogue: not held across the walk)
   bool any_act = false;
 #pragma unroll
-  for (int v = 0; v < VEC; ++v) any_act |= a.ws[w0 + v].active != 0;
+  for (int v = 0; v < VEC; ++v) any_act |= a.ws[w0 + woff<V>(v)].active != 0;
   const bool warp_act = __any_sync(0xffffffffu, any_act);
   R acc[VEC][2];
 #pragma unroll
@@ -920,15 +952,15 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
       C sg[VEC], be[VEC];
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
-        be[v] = to_c<R>(a.ws[w0 + v].beta);
-        sg[v] = a.sig[(w0 + v) & (a.mp - 1)];
+        be[v] = to_c<R>(a.ws[w0 + woff<V>(v)].beta);
+        sg[v] = a.sig[(w0 + woff<V>(v)) & (a.mp - 1)];
       }
 #pragma unroll
       for (int j = 0; j < G; ++j) {
         const int64_t i = g * G + j;
         if (i < a.n) {
           const size_t off = (size_t)i * a.W + w0;
-          if (!CHK(20, off + VEC - 1, (long long)a.n * a.W)) continue;
+          if (!CHK(20, off + woff<V>(VEC - 1), (long long)a.n * a.W)) continue;
           const Vec<R, VEC> rv = ldv<R, VEC>(a.r + off);
           Vec<R, VEC> pv, qv;
           if (!FRESH) {
@@ -957,6 +989,8 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
   spmm_tail<R, VEC>(a, acc, w_tile0, rb, tile, a.nrb);
 }
 
+#include "bricks.cuh"
+
 // ------------------------------------------------------------------------------ residual
 // Refinement step s >= 2 of the FP32 path: the FP64 residual of the accumulated correction
 //   R = r0 - (A - sigma B) D,   r0 = c_w gscale_c g,   D in FP64,
@@ -969,13 +1003,13 @@ __device__ __forceinline__ void cocg_residual_body(const CocgArgs<R> &a, const i
   using C = cx_t<R>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
-  const int w0 = w_tile0 + lane * VEC;
+  const int w0 = w_tile0 + lane_w<V>(lane);
   double2 sg[VEC], cf[VEC];
   int cidx[VEC];
   bool ok[VEC];
 #pragma unroll
   for (int v = 0; v < VEC; ++v) {
-    const int w = w0 + v;
+    const int w = w0 + woff<V>(v);
     sg[v] = a.sig64[w & (a.mp - 1)];
     cidx[v] = w / a.mp;
     ok[v] = cidx[v] < a.k;
@@ -1012,7 +1046,7 @@ __device__ __forceinline__ void cocg_residual_body(const CocgArgs<R> &a, const i
         const double2 *xr = a.D64 + (size_t)c * a.W + w0;
 #pragma unroll
         for (int v = 0; v < VEC; ++v) {
-          const double2 x = xr[v];
+          const double2 x = xr[woff<V>(v)];
           sa[v].x = fma(av, x.x, sa[v].x);
           sa[v].y = fma(av, x.y, sa[v].y);
           sb[v].x = fma(bv, x.x, sb[v].x);
@@ -1119,16 +1153,17 @@ __device__ __forceinline__ int batch_problem(const int *prefix, int P, int item)
   }
   return lo;
 }
-#define SLRF_BATCH_LOOP(BODY)                                               \
+#define SLRF_BATCH_LOOP(...)                                                \
   const int total = prefix[P];                                              \
   for (int item = blockIdx.x; item < total; item += gridDim.x) {            \
     const int pb = batch_problem(prefix, P, item);                          \
     const CocgArgs<R> &a = args[pb];                                        \
     const int local = item - prefix[pb];                                    \
-    BODY;                                                                   \
+    __VA_ARGS__;                                                            \
     __syncthreads();                                                        \
   }
-// (the batched path runs plain CSR only: lane width cocg_vec_csr<R>(), checked by the host)
+// (the batched path runs plain CSR, or in FP32 bricks: lane width cocg_vec_csr<R>(), checked by
+// the host)
 template <typename R>
 __global__ void __launch_bounds__(kThreads, (cocg_minb<R, cocg_vec_csr<R>()>())) cocg_init_batched(const CocgArgs<R> *args, const int *prefix, int P) {
   SLRF_BATCH_LOOP((cocg_init_body<R, cocg_vec_csr<R>()>(a, local % a.nrb, local / a.nrb)))
@@ -1144,6 +1179,20 @@ __global__ void __launch_bounds__(kThreads, (cocg_minb<R, cocg_vec_csr<R>()>()))
 template <typename R>
 __global__ void __launch_bounds__(kThreads, 2) cocg_residual_batched(const CocgArgs<R> *args, const int *prefix, int P) {
   SLRF_BATCH_LOOP((cocg_residual_body<R, cocg_vec_csr<R>()>(a, local % a.nrb, local / a.nrb)))
+}
+template <bool FRESH>
+__global__ void __launch_bounds__(kThreads, 2) cocg_brick_batched(const CocgArgs<float> *args, const int *prefix, int P) {
+  using R = float;
+  extern __shared__ __align__(128) unsigned char brick_smem[];
+  __shared__ __align__(8) uint64_t bar;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  unsigned phase = 0;
+  SLRF_BATCH_LOOP(
+      cocg_spmm_brick_body<FRESH>(a, local % a.bricks.blocks, local / a.bricks.blocks, brick_smem, &bar, phase))
 }
 #undef SLRF_BATCH_LOOP
 
@@ -1497,7 +1546,30 @@ template <typename R, int V, int G> static void spmm_grp_launch(const CocgArgs<R
   if (fresh) cocg_spmm_grp_kernel<R, V, G, false, true><<<grid_of(a), kThreads, grp_smem_bytes<R, G>(), st>>>(a);
   else cocg_spmm_grp_kernel<R, V, G, false, false><<<grid_of(a), kThreads, grp_smem_bytes<R, G>(), st>>>(a);
 }
+static void brick_launch(const CocgArgs<float> &a, cudaStream_t st, bool fresh) {
+  const dim3 grid((unsigned)a.bricks.blocks, (unsigned)(a.W / 64));
+  const int sm = brick_smem_bytes(a.bricks);
+  if (fresh) cocg_spmm_brick_kernel<true><<<grid, kThreads, sm, st>>>(a);
+  else cocg_spmm_brick_kernel<false><<<grid, kThreads, sm, st>>>(a);
+}
+int brick_group_size(int cmax, int &pad) {
+  pad = brick_pad(cmax);
+  return brick_group_bytes(cmax);
+}
+void brick_count(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int64_t ngroups,
+                 const int4 *groups, unsigned long long *most, cudaStream_t st) {
+  brick_count_kernel<<<(unsigned)((ngroups + 127) / 128), 128, 0, st>>>(ngroups, rowptr, col, valA, valB, groups, most);
+}
+void brick_build(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int count, int cmax,
+                 int pad, int group_bytes, int4 *groups, int *nrows, int *rows, unsigned char *rec, int *flag,
+                 unsigned long long *stats, cudaStream_t st) {
+  if (count > 0)
+    brick_build_kernel<<<count, 256, 0, st>>>(rowptr, col, valA, valB, cmax, pad, group_bytes, groups, nrows, rows, rec,
+                                              flag, stats);
+}
 template <typename R, int V> static void spmm_launch(const CocgArgs<R> &a, cudaStream_t st, bool fresh) {
+  if constexpr (sizeof(R) == 4)
+    if (a.bricks.count > 0) return brick_launch(a, st, fresh);
   switch (a.G) {
     case 2: spmm_grp_launch<R, V, 2>(a, st, fresh); return;
     case 3: spmm_grp_launch<R, V, 3>(a, st, fresh); return;
@@ -1552,7 +1624,7 @@ __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<float, kReal32Vec, G>
   extern __shared__ __align__(128) unsigned char grp_smem[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = (int)blockIdx.y * 64 * VEC + lane * 2 * VEC;  // the lane's pointer (see ldv): tile + 2 VEC lane
+  const int c0 = (int)blockIdx.y * 64 * VEC + 2 * lane_w<VEC>(lane);  // the lane's pointer (see ldv)
   // pair v of the lane (two real columns) sits at pair index 64 (v / 2) + 2 lane + v % 2 of the tile
   const int ct = (int)blockIdx.y * 64 * VEC;
   const int64_t gstride = (int64_t)a.nrb * kWarps;
@@ -1701,6 +1773,10 @@ void cocg_kernel_attrs() {
   grp_attrs<double, 2>();
   grp_attrs<double, 3>();
   grp_attrs<double, 4>();
+  cudaFuncSetAttribute(cocg_spmm_brick_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
+  cudaFuncSetAttribute(cocg_spmm_brick_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
+  cudaFuncSetAttribute(cocg_brick_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
+  cudaFuncSetAttribute(cocg_brick_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
   cudaGetLastError();
   done = true;
 }
@@ -1782,6 +1858,12 @@ template <typename R> void cocg_spmm_batched_launch(const CocgArgs<R> *args, con
                                                     bool fresh, cudaStream_t st) {
   if (fresh) cocg_spmm_batched<R, true><<<batch_grid(total), kThreads, 0, st>>>(args, prefix, P);
   else cocg_spmm_batched<R, false><<<batch_grid(total), kThreads, 0, st>>>(args, prefix, P);
+}
+void cocg_brick_batched_launch(const CocgArgs<float> *args, const int *prefix, int P, int total, int smem, bool fresh,
+                               cudaStream_t st) {
+  const int g = std::min(total, device_sm_count() * 2);
+  if (fresh) cocg_brick_batched<true><<<g, kThreads, smem, st>>>(args, prefix, P);
+  else cocg_brick_batched<false><<<g, kThreads, smem, st>>>(args, prefix, P);
 }
 template <typename R> void cocg_residual_batched_launch(const CocgArgs<R> *args, const int *prefix, int P, int total,
                                                         cudaStream_t st) {

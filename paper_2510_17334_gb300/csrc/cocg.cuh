@@ -22,6 +22,21 @@ constexpr int kThreads = 256;  // threads per COCG block (8 warps)
 constexpr int kWarps = kThreads / 32;
 constexpr int kNQ = 6;         // doubles per partial slot
 
+// Brick format of the FP32 SpMM (bricks.cuh); count 0: not in use.
+constexpr int kBrickRows = 192;    // staged rows of a brick, at most (their places fit a byte)
+constexpr int kBrickGroups = 16;   // row pairs of a brick, two per warp
+struct Bricks {
+  int count;        // bricks
+  int pad;          // record slots per group (values); the places follow
+  int group_bytes;  // bytes per group
+  int max_rows;     // staged rows of the largest brick
+  int blocks;       // row blocks per 64-entry column tile of a launch
+  const int4 *groups;  // [count][kBrickGroups]: first row, rows, records, place of the first row
+  const int *nrows;    // [count]
+  const int *rows;     // [count][kBrickRows]
+  const unsigned char *rec;  // [count][kBrickGroups * group_bytes]
+};
+
 template <typename R>
 struct CocgArgs {
   int64_t n;
@@ -77,6 +92,7 @@ struct CocgArgs {
   const int64_t *gptr;       // [ngroups + 1]
   const unsigned char *grec; // records, 16-byte aligned
   int bdiag;                 // 1: B-diagonal records (G = 3, see grec_col)
+  Bricks bricks;             // FP32: staged SpMM instead of the two above (count > 0)
   int *err;                  // 1: a bounded wait gave up (SLRF_ETIMEOUT); 2, 3: group records
                              // inconsistent; 4: update buffers missing (SLRF_EINVAL)
   // Jacobi preconditioner D = diag(A): the value arrays above are those of
@@ -131,6 +147,14 @@ template <typename R, int G, bool BD = false> __host__ __device__ constexpr int 
   return kWarps * 2 * grp_chunk<R, BD>() * grec_bytes<R, G, BD>();
 }
 
+// Dynamic shared memory of the brick SpMM (at least its reduction's scratch).
+inline int brick_smem_bytes(const Bricks &b) {
+  const int red = kWarps * 64 * 2 * (int)sizeof(double);
+  const int st = b.max_rows * 512 + kBrickGroups * b.group_bytes;
+  return st > red ? st : red;
+}
+constexpr int kBrickSmemMax = 112 * 1024;  // two blocks per SM
+
 // Final-update modes: how the last COCG update of a solve delivers its correction.
 // kAccU: an update of a solve without refinement adds its step to the accumulator (no d
 // array); kAccUEnd: the last one, which also writes U.
@@ -180,6 +204,9 @@ template <typename R> __host__ __device__ constexpr int cocg_vec_max() { return 
 template <typename R, int V> __host__ __device__ constexpr int cocg_minb() {
   return sizeof(R) == 8 ? 4 : (V >= 4 ? SLRF_F32_MINB4 : SLRF_F32_MINB);
 }
+template <typename R> inline int cocg_minb_rt(int vec) {
+  return sizeof(R) == 8 ? cocg_minb<R, 1>() : (vec >= 4 ? cocg_minb<R, 4>() : cocg_minb<R, 2>());
+}
 // Lane width and row length the kernels can use (else the launchers refuse, code 4).
 template <typename R> inline bool cocg_layout_ok(const CocgArgs<R> &a) {
   const bool v = sizeof(R) == 8 ? a.vec == 1 : (a.vec == 2 || a.vec == 4);
@@ -197,6 +224,10 @@ template <typename R> void cocg_update_batched_launch(const CocgArgs<R> *args, c
                                                       bool first, int fm, cudaStream_t st);
 template <typename R> void cocg_spmm_batched_launch(const CocgArgs<R> *args, const int *prefix, int P, int total,
                                                     bool fresh, cudaStream_t st);
+// SpMM of an FP32 batch whose problems all have bricks: prefix counts (row block, 64-entry tile)
+// items, smem the largest brick_smem_bytes.
+void cocg_brick_batched_launch(const CocgArgs<float> *args, const int *prefix, int P, int total, int smem, bool fresh,
+                               cudaStream_t st);
 template <typename R> void cocg_residual_batched_launch(const CocgArgs<R> *args, const int *prefix, int P, int total,
                                                         cudaStream_t st);
 
@@ -223,6 +254,14 @@ int grp_real64_ld(int k);
 void spmm_grp_real64(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *grec, int *err, int nrb,
                      const double *X, int ldx, int k, const double *xscale, double *x64, double *YA, double *YB,
                      int ldy, const double *yscale, cudaStream_t st);
+// Brick format: bytes of a group's record area, and the build (see bricks.cuh; groups holds
+// (first row, rows) on entry).
+int brick_group_size(int cmax, int &pad);
+void brick_count(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int64_t ngroups,
+                 const int4 *groups, unsigned long long *most, cudaStream_t st);
+void brick_build(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int count, int cmax,
+                 int pad, int group_bytes, int4 *groups, int *nrows, int *rows, unsigned char *rec, int *flag,
+                 unsigned long long *stats, cudaStream_t st);
 // Resident blocks per SM of the grouped SpMM of height G (after cocg_kernel_attrs; 0 on error).
 int grp_blocks_per_sm(int G, bool fp32, bool bd = false);
 

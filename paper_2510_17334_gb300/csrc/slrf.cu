@@ -94,6 +94,8 @@ struct slrf_ctx {
   int64_t rpb_tuned = 0;             // autotuned COCG rows per block (0 = default)
   int grp_bpsm = 0;                  // resident blocks per SM of the grouped SpMM in use
   int bdiag = 0;                     // the grouped records are B-diagonal (see grec_col)
+  Bricks bricks{};                   // mixed path: staged SpMM format (count 0: not in use)
+  bool batched = false;              // a problem of a batch: lane width 2 in FP32
   unsigned char *grec64 = nullptr;   // mixed path: FP64 B-diagonal records of the same groups
   double *x64 = nullptr;             // padded FP64 copy of a real block for the grouped FP64 products
   // real n x L blocks (ld = L)
@@ -256,7 +258,15 @@ static int group_counts(slrf_ctx *ctx, int G, std::vector<int> &cnt) {
   return e == cudaSuccess ? SLRF_OK : SLRF_ECUDA;
 }
 static int grec_size(int G, bool fp32) { return grec_bytes_rt(G, fp32); }
+static void drop_bricks(slrf_ctx *ctx) {
+  dfree(ctx, const_cast<int4 *>(ctx->bricks.groups));
+  dfree(ctx, const_cast<int *>(ctx->bricks.nrows));
+  dfree(ctx, const_cast<int *>(ctx->bricks.rows));
+  dfree(ctx, const_cast<unsigned char *>(ctx->bricks.rec));
+  ctx->bricks = Bricks{};
+}
 static void drop_groups(slrf_ctx *ctx) {
+  drop_bricks(ctx);
   dfree(ctx, ctx->gptr);
   dfree(ctx, ctx->grec);
   dfree(ctx, ctx->grec64);
@@ -362,8 +372,9 @@ static int build_groups(slrf_ctx *ctx, int G) {
 // Candidate G from the pattern.  FP64: the SpMM is bound by the FP64 pipe, so only groups
 // that add no zero products qualify (union x rows == entries), the largest such G.  FP32:
 // a cost per row, in units of one plain-CSR entry, fitted to GB300 timings of the 41^3
-// Laplacian (27 entries/row) and the 64x64x32 elasticity box (81): a record of a G-row
-// group costs about 1.2 + 0.25 G entries (the gather, the staged record, 8 G packed FMAs).
+// Laplacian (27 entries/row): CSR 1.50 ms, groups of 2, 3, 4 rows 1.21, 1.22, 1.29 ms, that is
+// 0.69 + 0.26 G entries for a record of a G-row group (the gather, the staged record, 8 G
+// packed FMAs).
 static int choose_group(slrf_ctx *ctx, int &G) {
   G = 1;
   double best = (double)ctx->nnz / ctx->n;
@@ -380,18 +391,151 @@ static int choose_group(slrf_ctx *ctx, int &G) {
       if (slots <= (double)ctx->nnz) { G = g; return SLRF_OK; }
       continue;
     }
-    const double cost = recs / ctx->n * (1.2 + 0.25 * g);
+    const double cost = recs / ctx->n * (0.69 + 0.26 * g);
     if (cost < best) { best = cost; G = g; }
   }
   return SLRF_OK;
 }
+// Strides of a mesh numbered line by line and plane by plane, from the columns of one row: the
+// offsets of its neighbours come in runs around +-1, the line stride and plane stride +- the
+// line stride; without such runs one line of everything.  Only the grouping of the rows into
+// bricks depends on it, and that is judged by the rows it stages.
+static void mesh_strides(const std::vector<int32_t> &cols, int64_t row, int64_t n, int64_t &line, int64_t &plane) {
+  line = plane = n;
+  std::vector<int64_t> pos;
+  for (int32_t c : cols)
+    if (c > row) pos.push_back(c - row);
+  std::vector<int64_t> centre;  // of the runs past the one that starts at 1
+  for (size_t i = 0; i < pos.size();) {
+    size_t e = i;
+    while (e + 1 < pos.size() && pos[e + 1] == pos[e] + 1) ++e;
+    if (pos[i] > 1) centre.push_back((pos[i] + pos[e]) / 2);
+    i = e + 1;
+  }
+  if (centre.empty() || centre[0] < 2) return;
+  line = centre[0];
+  if (centre.size() > 1) {
+    const int64_t p = centre[1 + (centre.size() - 1) / 2];
+    if (p % line == 0 && p > line) plane = p;
+  }
+}
+
+// Brick format of the FP32 SpMM (bricks.cuh): pairs of neighbouring rows gathered into bricks of
+// 4 x 4 x 2 rows (8 x 4 in a plane, 32 in a line).  Kept where the bricks stage at most 0.6 rows
+// per record they multiply (27-point pattern 0.25, 9-point 0.3, a line 0.53); without locality in
+// the numbering, or with rows too long for the shared memory of two blocks, the grouped or CSR
+// kernel stays.
+static int build_bricks(slrf_ctx *ctx) {
+  drop_bricks(ctx);
+  if (!ctx->mixed || ctx->grp != 2) return SLRF_OK;
+  const int64_t n = ctx->n;
+  std::vector<int64_t> rp((size_t)n + 1);
+  if (cudaMemcpyAsync(rp.data(), ctx->rowptr, rp.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->st) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(ctx->st) != cudaSuccess)
+    return SLRF_ECUDA;
+  // the longest row, the one next to the middle of several
+  int64_t row = n / 2, longest = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    const int64_t len = rp[i + 1] - rp[i];
+    if (len > longest || (len == longest && std::llabs(i - n / 2) < std::llabs(row - n / 2))) {
+      longest = len;
+      row = i;
+    }
+  }
+  if (longest < 1 || longest > 128) return SLRF_OK;
+  std::vector<int32_t> cols((size_t)longest);
+  if (cudaMemcpyAsync(cols.data(), ctx->col + rp[row], cols.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                      ctx->st) != cudaSuccess ||
+      cudaStreamSynchronize(ctx->st) != cudaSuccess)
+    return SLRF_ECUDA;
+  int64_t line, plane;
+  mesh_strides(cols, row, n, line, plane);
+  const bool d1 = line >= n, d2 = !d1 && plane >= n;
+  const int64_t bx = d1 ? 32 : (d2 ? 8 : 4), by = d1 ? 1 : 4, bz = d1 || d2 ? 1 : 2;  // 2 kBrickGroups rows
+  std::vector<int4> groups;
+  groups.reserve((size_t)(n * 5 / 8 + kBrickGroups));
+  const int64_t ny = (plane + line - 1) / line, nz = (n + plane - 1) / plane;
+  for (int64_t z0 = 0; z0 < nz; z0 += bz)
+    for (int64_t y0 = 0; y0 < ny; y0 += by)
+      for (int64_t x0 = 0; x0 < line; x0 += bx) {
+        const size_t first = groups.size();
+        for (int64_t z = z0; z < std::min(nz, z0 + bz); ++z)
+          for (int64_t y = y0; y < std::min(ny, y0 + by); ++y)
+            for (int64_t x = x0; x < std::min(line, x0 + bx); x += 2) {
+              const int64_t i = x + line * y + plane * z;
+              if (i < n) groups.push_back(make_int4((int)i, x + 1 < line && i + 1 < n ? 2 : 1, 0, 0));
+            }
+        if (groups.size() == first) continue;
+        while ((groups.size() - first) % kBrickGroups) groups.push_back(make_int4(0, 0, 0, 0));
+      }
+  Bricks B{};
+  B.count = (int)(groups.size() / kBrickGroups);
+  auto give_up = [&](int rc) {
+    ctx->bricks = B;
+    drop_bricks(ctx);
+    return rc;
+  };
+  int4 *dg = nullptr;
+  int *dn = nullptr, *dr = nullptr;
+  unsigned char *rec = nullptr;
+  unsigned long long *stats = nullptr;  // staged rows, records, largest brick, longest group, flag
+  int rc;
+  if ((rc = dalloc(ctx, &dg, groups.size())) != SLRF_OK) return rc;
+  B.groups = dg;
+  if ((rc = dalloc(ctx, &dn, (size_t)B.count)) != SLRF_OK) return give_up(rc);
+  B.nrows = dn;
+  if ((rc = dalloc(ctx, &dr, (size_t)B.count * kBrickRows)) != SLRF_OK) return give_up(rc);
+  B.rows = dr;
+  if ((rc = dalloc(ctx, &stats, 5)) != SLRF_OK) return give_up(rc);
+  unsigned long long h[5] = {};
+  cudaMemsetAsync(stats, 0, 5 * sizeof(unsigned long long), ctx->st);
+  cudaMemcpyAsync(dg, groups.data(), groups.size() * sizeof(int4), cudaMemcpyHostToDevice, ctx->st);
+  brick_count(ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), (int64_t)groups.size(), dg, stats + 3, ctx->st);
+  cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, ctx->st);
+  if (cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+    dfree(ctx, stats);
+    return give_up(SLRF_ECUDA);
+  }
+  const int cmax = (int)h[3];
+  bool fit = cmax >= 1 && kBrickGroups * cmax <= 2048;
+  if (fit) {
+    B.group_bytes = brick_group_size(cmax, B.pad);
+    rc = dalloc(ctx, &rec, (size_t)B.count * kBrickGroups * B.group_bytes);
+    if (rc != SLRF_OK) {
+      dfree(ctx, stats);
+      return give_up(rc);
+    }
+    B.rec = rec;
+    brick_build(ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), B.count, cmax, B.pad, B.group_bytes, dg, dn,
+                dr, rec, reinterpret_cast<int *>(stats + 4), stats, ctx->st);
+    cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, ctx->st);
+    if (cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+      dfree(ctx, stats);
+      return give_up(SLRF_ECUDA);
+    }
+    B.max_rows = (int)h[2];
+    fit = h[4] == 0 && (double)h[0] <= 0.6 * (double)h[1] && brick_smem_bytes(B) <= kBrickSmemMax;
+  }
+  dfree(ctx, stats);
+  if (!fit) return give_up(SLRF_OK);
+  ctx->bricks = B;
+  ctx->vec = cocg_vec_csr<float>();  // 64-entry tiles
+  return SLRF_OK;
+}
+
 static int setup_groups(slrf_ctx *ctx) {
   int G = ctx->o.group;
   if (G == 0) {
     int rc = choose_group(ctx, G);
     if (rc != SLRF_OK) return rc;
   }
-  return build_groups(ctx, G);
+  int rc = build_groups(ctx, G);
+  if (rc != SLRF_OK) return rc;
+  if (ctx->o.group == 0 && (rc = build_bricks(ctx)) != SLRF_OK) return rc;
+  // the batched kernels run bricks or plain CSR, at the CSR lane width
+  if (ctx->batched && ctx->bricks.count == 0) drop_groups(ctx);
+  return SLRF_OK;
 }
 
 // ----------------------------------------------------------------------------- filter
@@ -443,24 +587,26 @@ static void real_products64(slrf_ctx *ctx, const double *X, int ldx, int k, doub
 // reduction, arrival at the tile's counter) and its rows' share of the SM, and a tile's last
 // block sums one slot per row block; for small problems the split that fills the row_blocks()
 // limit (16 rows a block) is mostly that latency.  The model, in microseconds, is fitted to
-// timings of GB300 between n = 930 and 68,921: a block 6 + 0.13 a row, four at a time on an SM;
+// timings of GB300 between n = 930 and 68,921: a block 6 + 0.13 a row, per_sm at a time on an SM;
 // the SM's throughput 0.02 + 0.0036 per stored entry and row in FP32, 0.1 + 0.035 in FP64 (its
-// FP64 pipe); 0.05 per row block in the last block's sum.  At most 128 rows, so that the
-// gathered rows of the blocks in flight (4 an SM, 512 bytes a row) stay within a third of L2.
+// FP64 pipe); 0.05 per row block in the last block's sum.  At most `most` rows: 128 where the
+// SpMM uses them, so that the gathered rows of the blocks in flight (4 an SM, 512 bytes a row)
+// stay within a third of L2, 512 where only the streaming launches do.
 // `row_tiles`: rows x column tiles of the launch (over all problems of an FP32 batch).
 // FP32, It_max 8, 20^3 nodes, 32 columns: 16 rows a block 1.46 ms, 48 rows 0.89 ms; a solve of
 // 21 x 20 x 19 nodes, block 100: 182 -> 136 ms; 41^3 nodes, 160 columns: 120 rows 18.3 ms,
 // 128 rows 18.0 ms, 256 rows 20.1 ms.
-static int64_t csr_rows(const slrf_ctx *ctx, double row_tiles, bool fp32) {
+static int64_t csr_rows(const slrf_ctx *ctx, double row_tiles, bool fp32, int per_sm, int64_t most) {
   const int64_t sms = ctx->sm_count, n = ctx->n;
   const double nnz_row = (double)ctx->nnz / n, tiles = std::max(1.0, row_tiles / n);
   const double thr = fp32 ? 0.02 + 0.0036 * nnz_row : 0.1 + 0.035 * nnz_row;
   const int64_t least = (n + 4 * sms - 1) / (4 * sms);  // the partial sums hold 4 row blocks per SM
-  int64_t best = (least + kWarps - 1) / kWarps * kWarps;
+  int64_t best = std::max<int64_t>(16, (least + kWarps - 1) / kWarps * kWarps);
   double best_cost = 1e300;
-  for (int64_t r = best; r <= std::max<int64_t>(best, 128); r += kWarps) {
+  for (int64_t r = best; r <= std::max<int64_t>(least, most); r += kWarps) {
     const double nrb = (double)((n + r - 1) / r), blocks = std::ceil(nrb * tiles);
-    const double cost = std::ceil(blocks / sms) * r * thr + std::ceil(blocks / (4 * sms)) * (6.0 + 0.13 * r) + 0.05 * nrb;
+    const double cost = std::ceil(blocks / sms) * r * thr +
+                        std::ceil(blocks / (per_sm * sms)) * (6.0 + 0.13 * r) + 0.05 * nrb;
     if (cost < best_cost) { best_cost = cost; best = r; }
   }
   return best;
@@ -478,10 +624,11 @@ static CocgArgs<R> build_cocg_args(slrf_ctx *ctx, const double *X, int ldx, int 
   const int64_t rblocks = row_blocks(ctx);
   int64_t rpb = std::max<int64_t>(16, (ctx->n + rblocks - 1) / rblocks);
   if (ctx->rpb_tuned > 0) rpb = std::max<int64_t>(rpb, ctx->rpb_tuned);
-  else if (ctx->grp == 1)
-    rpb = csr_rows(ctx, row_tiles > 0.0 ? row_tiles : (double)ctx->n * (W / (32 * vec)), sizeof(R) == 4);
+  else if (ctx->grp == 1 || ctx->bricks.count > 0)
+    rpb = csr_rows(ctx, row_tiles > 0.0 ? row_tiles : (double)ctx->n * (W / (32 * vec)), sizeof(R) == 4,
+                   cocg_minb_rt<R>(vec), ctx->bricks.count > 0 ? 512 : 128);
   // whole groups per row block, the same number for every warp of the block
-  const int64_t unit = (int64_t)ctx->grp * kWarps;
+  const int64_t unit = ctx->bricks.count > 0 ? kWarps : (int64_t)ctx->grp * kWarps;
   rpb = (rpb + unit - 1) / unit * unit;
   const int nrb = (int)((ctx->n + rpb - 1) / rpb);
   CocgArgs<R> a{};
@@ -498,6 +645,18 @@ static CocgArgs<R> build_cocg_args(slrf_ctx *ctx, const double *X, int ldx, int 
   a.gptr = ctx->gptr;
   a.grec = ctx->grec;
   a.bdiag = ctx->bdiag;
+  if (sizeof(R) == 4 && ctx->bricks.count > 0) {
+    // Two blocks per SM over the tiles in flight, every block about as many bricks as the
+    // others.  The tiles go in waves whose gathered rows (n x 512 bytes a tile) stay within 40 MB
+    // of L2.
+    a.bricks = ctx->bricks;
+    const int64_t slots = 2 * (int64_t)ctx->sm_count, T = W / 64;
+    const int64_t cap = std::max<int64_t>(1, (40 << 20) / (ctx->n * 512));
+    const int64_t waves = (T + cap - 1) / cap, tiles = (T + waves - 1) / waves;
+    const int64_t nb = std::min<int64_t>(ctx->bricks.count, std::max<int64_t>(1, slots / tiles));
+    const int64_t per = (ctx->bricks.count + nb - 1) / nb;
+    a.bricks.blocks = (int)((ctx->bricks.count + per - 1) / per);
+  }
   a.err = ctx->iflags + 15;
   a.dsc = ctx->dsc;
   a.uacc = ctx->uacc;
@@ -550,7 +709,7 @@ static int run_cocg(slrf_ctx *ctx, const double *X, int ldx, int k, const double
   // the update of the other (cocg_dual); each group still alternates update and SpMM in
   // order.  Measured on the 41^3 workload: -3 % filter time in FP32; in FP64 both kernels
   // load the FP64 pipe (the update does ~11 FP64 FMAs per entry), so there it is not used.
-  const bool dual_ok = sizeof(R) == 4 && T >= 2 && itm >= 2 && ctx->grp == 1;
+  const bool dual_ok = sizeof(R) == 4 && T >= 2 && itm >= 2 && ctx->grp == 1 && ctx->bricks.count == 0;
   ctx->launches += 2 * itm + 1 + (sizeof(R) == 4 ? 3 : 0) + (int64_t)(nref - 1) * (2 * itm + 1) +
                    (dual_ok && tm == nullptr ? nref : 0);
   // one launch sequence for the graph, the direct and the timed path; `kind` tags each
@@ -726,24 +885,37 @@ static int autotune_rows(slrf_ctx *ctx) {
     return SLRF_OK;
   };
   float best = 1e30f, t = 0;
-  if (ctx->o.group == 0) {
+  if (ctx->o.group == 0 && !ctx->batched) {
     // group height: plain CSR and every grouped format the precision admits (FP64: the
     // no-fill height the pattern model found, if any; FP32: 2, 3 and 4)
     const int g_model = ctx->grp;
     int best_g = 1;
+    bool best_bricks = false;
     for (int g = 1; g <= 4; ++g) {
       if (g > 1 && !ctx->mixed && g != g_model) continue;
       if ((rc = build_groups(ctx, g)) != SLRF_OK) break;
       ctx->rpb_tuned = 0;
       if ((rc = time_spmm(t)) != SLRF_OK) break;
-      if (t < best) { best = t; best_g = g; }
+      if (t < best) { best = t; best_g = g; best_bricks = false; }
+      if ((rc = build_bricks(ctx)) != SLRF_OK) break;
+      if (ctx->bricks.count == 0) continue;
+      if ((rc = time_spmm(t)) != SLRF_OK) break;
+      if (t < best) { best = t; best_g = g; best_bricks = true; }
     }
     if (rc == SLRF_OK) rc = build_groups(ctx, best_g);
+    if (rc == SLRF_OK && best_bricks) rc = build_bricks(ctx);
     if (rc != SLRF_OK) {
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
       return rc;
     }
+  }
+  if (ctx->bricks.count > 0) {  // the rows per block only split the update launches
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    ctx->rpb_tuned = 0;
+    CKL();
+    return SLRF_OK;
   }
   const int64_t base = base_rows();
   const int64_t cand[] = {base, 32, 64, 128, 256};
@@ -888,9 +1060,9 @@ struct slrf_batch {
   std::vector<cudaEvent_t> ev_p;
   bool mixed = false;
   void *dargs = nullptr, *hargs = nullptr;
-  int *dprefix = nullptr, *hprefix = nullptr;
+  int *dprefix = nullptr, *hprefix = nullptr;  // item offsets, then those of the brick SpMM
   cudaGraphExec_t gexec = nullptr;
-  int g_P = -1, g_total = -1, g_itm = -1;
+  int g_P = -1, g_total = -1, g_itm = -1, g_btotal = -1, g_bsmem = -1;
 };
 
 static void batch_free(slrf_batch *b) {
@@ -909,22 +1081,28 @@ static void batch_free(slrf_batch *b) {
 }
 
 // One persistent batched COCG pass over the active problems (args/prefix already on the
-// device): init, then refine_max x (It_max updates and SpMMs), on the batch stream.
+// device): init, then refine_max x (It_max updates and SpMMs), on the batch stream.  btotal > 0:
+// the SpMM runs on bricks (that many items).
 template <typename R>
-static void batch_cocg(slrf_batch *b, int P, int total, int nref, int itm, cudaStream_t s) {
+static void batch_cocg(slrf_batch *b, int P, int total, int btotal, int bsmem, int nref, int itm, cudaStream_t s) {
   const CocgArgs<R> *args = reinterpret_cast<const CocgArgs<R> *>(b->dargs);
   const int *pre = b->dprefix;
+  auto spmm = [&](bool fresh) {
+    if constexpr (sizeof(R) == 4)
+      if (btotal > 0) return cocg_brick_batched_launch(args, b->dprefix + b->P + 1, P, btotal, bsmem, fresh, s);
+    cocg_spmm_batched_launch<R>(args, pre, P, total, fresh, s);
+  };
   cocg_init_batched_launch<R>(args, pre, P, total, s);
   for (int step = 1; step <= nref; ++step) {
     if (step > 1) {
       if constexpr (sizeof(R) == 4) cocg_residual_batched_launch<R>(args, pre, P, total, s);
-      cocg_spmm_batched_launch<R>(args, pre, P, total, true, s);
+      spmm(true);
     }
     int fm_mid, fm_last;
     update_modes<R>(nref, step, fm_mid, fm_last);
     for (int it = 1; it <= itm; ++it) {
       cocg_update_batched_launch<R>(args, pre, P, total, it == 1, it == itm ? fm_last : fm_mid, s);
-      if (it < itm) cocg_spmm_batched_launch<R>(args, pre, P, total, false, s);
+      if (it < itm) spmm(false);
     }
   }
 }
@@ -951,7 +1129,7 @@ static int batch_outer_filter(slrf_batch *b, const std::vector<int> &act, const 
     if (rc != SLRF_OK) return rc;
     ha[i] = build_cocg_args<R>(c, c->V, c->L, k, c->U, c->L, nref, row_tiles);
     ha[i].it_cap = c->o.it_adapt ? c->it_cur : 0;  // per-problem It_max inside the shared loop
-    if (ha[i].vec != vec || ha[i].G != 1) return SLRF_EINVAL;  // the batched setup forces group = 1
+    if (ha[i].vec != vec || (ha[i].G != 1 && ha[i].bricks.count == 0)) return SLRF_EINVAL;  // see setup_groups
     for (int step = 1; step <= nref; ++step) {  // the batched kernels read these buffers unchecked
       int fm_mid, fm_last;
       update_modes<R>(nref, step, fm_mid, fm_last);
@@ -966,16 +1144,38 @@ static int batch_outer_filter(slrf_batch *b, const std::vector<int> &act, const 
     CK(cudaEventRecord(b->ev_p[act[i]], c->st));
     CK(cudaStreamWaitEvent(b->st, b->ev_p[act[i]], 0));
   }
+  // bricks, when every problem has them: about two items per resident block, each of as many
+  // bricks as the others
+  int btotal = 0, bsmem = 0;
+  if (sizeof(R) == 4) {
+    double bricks = 0.0;
+    bool all = true;
+    for (int i = 0; i < P; ++i) {
+      all = all && ha[i].bricks.count > 0;
+      bricks += (double)ha[i].bricks.count * (ha[i].W / 64);
+    }
+    const int64_t per = std::max<int64_t>(1, (int64_t)std::ceil(bricks / (4.0 * b->c[act[0]]->sm_count)));
+    int *const pre = b->hprefix + b->P + 1;
+    pre[0] = 0;
+    for (int i = 0; all && i < P; ++i) {
+      Bricks &B = ha[i].bricks;
+      B.blocks = (int)((B.count + per - 1) / per);
+      btotal += B.blocks * (ha[i].W / 64);
+      bsmem = std::max(bsmem, brick_smem_bytes(B));
+      pre[i + 1] = btotal;
+    }
+  }
   CK(cudaMemcpyAsync(b->dargs, b->hargs, P * sizeof(CocgArgs<R>), cudaMemcpyHostToDevice, b->st));
-  CK(cudaMemcpyAsync(b->dprefix, b->hprefix, (P + 1) * sizeof(int), cudaMemcpyHostToDevice, b->st));
+  CK(cudaMemcpyAsync(b->dprefix, b->hprefix, 2 * (b->P + 1) * sizeof(int), cudaMemcpyHostToDevice, b->st));
   launches += 1 + (int64_t)nref * (2 * itm - 1) + (nref - 1) * (sizeof(R) == 4 ? 2 : 1);
   CK(cudaEventRecord(b->ev_f0, b->st));
   if (b->c[act[0]]->o.use_graph) {
-    if (!(b->gexec && b->g_P == P && b->g_total == total && b->g_itm == itm)) {
+    if (!(b->gexec && b->g_P == P && b->g_total == total && b->g_itm == itm && b->g_btotal == btotal &&
+          b->g_bsmem == bsmem)) {
       if (b->gexec) { cudaGraphExecDestroy(b->gexec); b->gexec = nullptr; }
       cudaGraph_t g;
       CK(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
-      batch_cocg<R>(b, P, total, nref, itm, b->st);
+      batch_cocg<R>(b, P, total, btotal, bsmem, nref, itm, b->st);
       CK(cudaStreamEndCapture(b->st, &g));
       cudaError_t e = cudaGraphInstantiate(&b->gexec, g, 0);
       cudaGraphDestroy(g);
@@ -983,10 +1183,12 @@ static int batch_outer_filter(slrf_batch *b, const std::vector<int> &act, const 
       b->g_P = P;
       b->g_total = total;
       b->g_itm = itm;
+      b->g_btotal = btotal;
+      b->g_bsmem = bsmem;
     }
     CK(cudaGraphLaunch(b->gexec, b->st));
   } else {
-    batch_cocg<R>(b, P, total, nref, itm, b->st);
+    batch_cocg<R>(b, P, total, btotal, bsmem, nref, itm, b->st);
   }
   if (cudaGetLastError() != cudaSuccess) return SLRF_ECUDA;
   CK(cudaEventRecord(b->ev_f1, b->st));
@@ -1127,8 +1329,10 @@ void slrf_destroy(slrf_ctx *ctx) {
   delete ctx;
 }
 
-int slrf_setup(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int block_L, const slrf_opts *opts,
-               void *stream) {
+}  // extern "C"
+
+static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int block_L, const slrf_opts *opts,
+                      void *stream, bool batched) {
   if (!out) return SLRF_EINVAL;
   *out = nullptr;
   if (!pc || !pc->rowptr || !pc->col || !pc->valA || !pc->valB || pc->n < 1 || pc->nnz < 1) return SLRF_EINVAL;
@@ -1170,6 +1374,7 @@ int slrf_setup(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int block_
   ctx->m = o.m;
   ctx->mp = pow2_at_least(o.m);
   ctx->mixed = o.precision == 1;
+  ctx->batched = batched;
   ctx->vec = ctx->mixed ? cocg_vec_csr<float>() : cocg_vec_csr<double>();  // until groups are built
   const int64_t n = ctx->n;
   const int L = block_L;
@@ -1338,6 +1543,13 @@ int slrf_setup(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int block_
   if (cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(SLRF_ECUDA);
   *out = ctx;
   return SLRF_OK;
+}
+
+extern "C" {
+
+int slrf_setup(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int block_L, const slrf_opts *opts,
+               void *stream) {
+  return setup_impl(out, pc, gamma, block_L, opts, stream, false);
 }
 
 int slrf_get_poles(slrf_ctx *ctx, int *m_out, double *sigma, double *w) {
@@ -1653,13 +1865,14 @@ int slrf_setup_batched(slrf_batch **out, int P, const slrf_csr_pair *pencils, co
   b->ust = (cudaStream_t)stream;
   b->c.assign(P, nullptr);
   b->ev_p.assign(P, nullptr);
-  // the persistent batched launches gather through the plain CSR pattern of each problem
+  // the persistent batched launches run bricks (FP32, where every active problem has them) or
+  // gather through the plain CSR pattern of each problem
   slrf_opts ob;
   if (opts) ob = *opts;
   else slrf_opts_default(&ob);
-  ob.group = 1;
+  ob.group = ob.precision == 1 ? 0 : 1;
   for (int p = 0; p < P; ++p) {
-    const int rc = slrf_setup(&b->c[p], &pencils[p], gammas[p], blocks[p], &ob, stream);
+    const int rc = setup_impl(&b->c[p], &pencils[p], gammas[p], blocks[p], &ob, stream, true);
     if (rc != SLRF_OK) {
       batch_free(b);
       return rc;
@@ -1672,8 +1885,8 @@ int slrf_setup_batched(slrf_batch **out, int P, const slrf_csr_pair *pencils, co
       cudaEventCreateWithFlags(&b->ev_b, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreate(&b->ev_t0) != cudaSuccess || cudaEventCreate(&b->ev_t1) != cudaSuccess ||
       cudaEventCreate(&b->ev_f0) != cudaSuccess || cudaEventCreate(&b->ev_f1) != cudaSuccess ||
-      cudaMalloc(&b->dargs, P * asz) != cudaSuccess || cudaMalloc(&b->dprefix, (P + 1) * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&b->hargs, P * asz) != cudaSuccess || cudaMallocHost(&b->hprefix, (P + 1) * sizeof(int)) != cudaSuccess) {
+      cudaMalloc(&b->dargs, P * asz) != cudaSuccess || cudaMalloc(&b->dprefix, 2 * (P + 1) * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&b->hargs, P * asz) != cudaSuccess || cudaMallocHost(&b->hprefix, 2 * (P + 1) * sizeof(int)) != cudaSuccess) {
     batch_free(b);
     return SLRF_ECUDA;
   }
