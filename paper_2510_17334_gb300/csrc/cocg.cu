@@ -731,12 +731,16 @@ __device__ __forceinline__ void cocg_spmm_body(const CocgArgs<R> &a, const int r
 // (2 s, then *err and a drain of the outstanding copies); inconsistent offsets set *err = 2
 // (and, with SLRF_GRP_COLCHECK, a record column out of range *err = 3, gathering row 0; by
 // default the columns are checked once when the records are built).
-template <typename R, int V, int G, bool BD, typename Epi>
+// U > 0 (FP64 B-diagonal records): the lane takes U single columns instead, column u of the
+// gathered row at xlane + c * xbytes + xo[u], and sa, sb hold U reals per row.
+template <typename R, int V, int G, bool BD, int U = 0, typename Epi>
 __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *__restrict__ gptr,
                                          const unsigned char *__restrict__ grec, int *err, const int64_t nx,
                                          const int64_t gfirst, const int64_t gstride, const char *xlane,
-                                         const unsigned xbytes, unsigned char *sbuf, uint64_t *bar, Epi &&epi) {
-  constexpr int VEC = V;
+                                         const unsigned xbytes, unsigned char *sbuf, uint64_t *bar, Epi &&epi,
+                                         const int *xo = nullptr) {
+  static_assert(U == 0 || (BD && sizeof(R) == 8), "single columns: FP64 B-diagonal records");
+  constexpr int VEC = U > 0 ? U : V;
   constexpr int RS = grec_bytes<R, G, BD>();
   constexpr int CH = grp_chunk<R, BD>();
   static_assert(!BD || (G == 3 && CH % 3 == 0), "B-diagonal records: 3-row groups, whole triples per chunk");
@@ -790,11 +794,12 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
   uint32_t ph0 = 0, ph1 = 0;
   int b = 0;
   bool failed = false;
-  C sa[G][VEC], sb[G][VEC];
+  using S = std::conditional_t<(U > 0), double, C>;
+  S sa[G][VEC], sb[G][VEC];
 #pragma unroll
   for (int j = 0; j < G; ++j)
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) { sa[j][v] = cmake<C>(0, 0); sb[j][v] = cmake<C>(0, 0); }
+    for (int v = 0; v < VEC; ++v) sa[j][v] = sb[j][v] = S{};
   while (cg < gb1) {
     if (!mbar_wait(bar + b, b ? ph1 : ph0, err, 1)) { failed = true; break; }
     if (b) ph1 ^= 1u; else ph0 ^= 1u;
@@ -810,7 +815,21 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
         for (int d = 0; d < 3; ++d) {
           const unsigned char *rp = rb_ + (t + d) * RS;
           const int c = *reinterpret_cast<const int *>(rp + grec_col<R, G, true>());
-          const Vec<R, VEC> x = ldv<R, VEC>(reinterpret_cast<const C *>(xlane + (unsigned long long)(unsigned)c * xbytes));
+          const char *const xc = xlane + (unsigned long long)(unsigned)c * xbytes;
+          if constexpr (U > 0) {
+            const double2 r01 = reinterpret_cast<const double2 *>(rp)[0];  // a0, a1
+            const double2 r23 = reinterpret_cast<const double2 *>(rp)[1];  // a2, b
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const double x = *reinterpret_cast<const double *>(xc + xo[u]);
+              sa[0][u] = fma(r01.x, x, sa[0][u]);
+              sa[1][u] = fma(r01.y, x, sa[1][u]);
+              sa[2][u] = fma(r23.x, x, sa[2][u]);
+              sb[d][u] = fma(r23.y, x, sb[d][u]);
+            }
+            continue;
+          } else {
+          const Vec<R, VEC> x = ldv<R, VEC>(reinterpret_cast<const C *>(xc));
           if constexpr (sizeof(R) == 4) {
             const float4 r4 = *reinterpret_cast<const float4 *>(rp);  // a0, a1, a2, b
             const float2 a0 = make_float2(r4.x, r4.x), a1 = make_float2(r4.y, r4.y), a2 = make_float2(r4.z, r4.z);
@@ -837,9 +856,10 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
               sb[d][v].y = fma(r23.y, x.z[v].y, sb[d][v].y);
             }
           }
+          }
         }
       }
-    } else {
+    } else if constexpr (U == 0) {
 #pragma unroll kGrpUnroll
     for (int t = 0; t < cnt; ++t) {
       const unsigned char *rp = rb_ + t * RS;
@@ -892,7 +912,7 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
 #pragma unroll
       for (int j = 0; j < G; ++j)
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) { sa[j][v] = cmake<C>(0, 0); sb[j][v] = cmake<C>(0, 0); }
+        for (int v = 0; v < VEC; ++v) sa[j][v] = sb[j][v] = S{};
     }
     __syncwarp();
     // stage the item after next into the buffer just read
@@ -1672,10 +1692,12 @@ void spmm_grp_real32(int64_t n, int G, int64_t ngroups, const int64_t *gptr, con
   }
 }
 
-// FP64 real products through FP64 B-diagonal records (3-row groups): a lane takes one
-// double2 -- two adjacent real columns -- of the padded FP64 copy x64, so a warp covers 64
-// columns per tile and the FMAs are those of the complex FP64 SpMM (A and B products per
-// gathered row: 3 + 1).  Output row i is multiplied by yscale[i] (null: 1).
+// FP64 real products through FP64 B-diagonal records (3-row groups), bound by the FP64 pipe: 4
+// multiply-adds (3 A, 1 B) per record and column, 16 clocks of the SM for 32 columns.  A lane
+// takes U columns 32 apart (U of 1..4 with the fewest padded columns in all), so only the last
+// 32 of k are padded: 96 columns of the 32 x 32 x 16 box 1.03 ms as two tiles of 64 double2
+// lanes -> 0.76 ms.  X is read in place unless its rows have to be scaled.  Output row i is
+// multiplied by yscale[i] (null: 1).
 struct GrpReal64 {
   int64_t n, ngroups;
   const int64_t *gptr;
@@ -1693,50 +1715,67 @@ int grp_real64_ld(int k) { return (k + 63) / 64 * 64; }
 __global__ void to_f64_scaled_kernel(int64_t n, int k, const double *__restrict__ X, int ldx,
                                      const double *__restrict__ s, double *__restrict__ Y, int ldy) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * ldy) return;
-  const int64_t i = t / ldy;
-  const int c = (int)(t - i * ldy);
-  Y[t] = c < k ? (s != nullptr ? X[i * ldx + c] * s[i] : X[i * ldx + c]) : 0.0;
+  if (t >= n * k) return;
+  const int64_t i = t / k;
+  const int c = (int)(t - i * k);
+  Y[i * ldy + c] = X[i * ldx + c] * s[i];
 }
+template <int U>
 __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<double, 1, 3>())) spmm_grp_real64_kernel(const GrpReal64 a) {
   constexpr int RS = grec_bytes<double, 3, true>();
   extern __shared__ __align__(128) unsigned char grp_smem[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = (int)blockIdx.y * 64 + 2 * lane;  // this lane's two real columns
+  const int c0 = (int)blockIdx.y * (32 * U) + lane;
+  int xo[U];  // byte offsets of the lane's columns (past the last one: the last one again)
+#pragma unroll
+  for (int u = 0; u < U; ++u) xo[u] = 8 * (c0 + 32 * u < a.k ? c0 + 32 * u : a.k - 1);
   const int64_t gstride = (int64_t)a.nrb * kWarps;
   const int64_t gfirst = (int64_t)blockIdx.x * kWarps + warp;
   if (gfirst >= a.ngroups) return;  // warp-uniform; the kernel has no block-wide barrier
-  auto epi = [&](int64_t g, const double2 (&sa)[3][1], const double2 (&sb)[3][1]) {
+  auto epi = [&](int64_t g, const double (&sa)[3][U], const double (&sb)[3][U]) {
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int64_t i = g * 3 + j;
       if (i >= a.n) continue;
-      const double ys = a.yscale != nullptr ? a.yscale[i] : 1.0;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int c = c0 + e;
-        if (c < a.k) {
-          if (a.YA) a.YA[(size_t)i * a.ldy + c] = ys * (e ? sa[j][0].y : sa[j][0].x);
-          if (a.YB) a.YB[(size_t)i * a.ldy + c] = ys * (e ? sb[j][0].y : sb[j][0].x);
-        }
+      for (int u = 0; u < U; ++u) {
+        const int c = c0 + 32 * u;
+        if (c >= a.k) continue;
+        const double ya = a.yscale != nullptr ? a.yscale[i] * sa[j][u] : sa[j][u];
+        const double yb = a.yscale != nullptr ? a.yscale[i] * sb[j][u] : sb[j][u];
+        if (a.YA) a.YA[(size_t)i * a.ldy + c] = ya;
+        if (a.YB) a.YB[(size_t)i * a.ldy + c] = yb;
       }
     }
   };
-  grp_walk<double, 1, 3, true>(a.ngroups, a.gptr, a.grec, a.err, a.n, gfirst, gstride,
-                               reinterpret_cast<const char *>(a.x + c0), (unsigned)a.ldx * 8u,
-                               grp_smem + (size_t)warp * 2 * grp_chunk<double, true>() * RS, s_bar[warp], epi);
+  grp_walk<double, 1, 3, true, U>(a.ngroups, a.gptr, a.grec, a.err, a.n, gfirst, gstride,
+                                  reinterpret_cast<const char *>(a.x), (unsigned)a.ldx * 8u,
+                                  grp_smem + (size_t)warp * 2 * grp_chunk<double, true>() * RS, s_bar[warp], epi, xo);
 }
 void spmm_grp_real64(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *grec, int *err, int nrb,
                      const double *X, int ldx, int k, const double *xscale, double *x64, double *YA, double *YB,
                      int ldy, const double *yscale, cudaStream_t st) {
   if (n <= 0 || k <= 0 || nrb <= 0) return;
-  const int ld64 = grp_real64_ld(k);
-  const int64_t tot = n * ld64;
-  to_f64_scaled_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n, k, X, ldx, xscale, x64, ld64);
-  GrpReal64 a{n, ngroups, gptr, grec, err, nrb, x64, ld64, k, YA, YB, ldy, yscale};
-  const dim3 grid((unsigned)nrb, (unsigned)(ld64 / 64));
-  spmm_grp_real64_kernel<<<grid, kThreads, grp_smem_bytes<double, 3, true>(), st>>>(a);
+  if (xscale != nullptr) {
+    const int64_t tot = n * k;
+    to_f64_scaled_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n, k, X, ldx, xscale, x64, k);
+    X = x64;
+    ldx = k;
+  }
+  GrpReal64 a{n, ngroups, gptr, grec, err, nrb, X, ldx, k, YA, YB, ldy, yscale};
+  const int groups = (k + 31) / 32;
+  int U = 1, padded = groups;
+  for (int u = 2; u <= 4; ++u)
+    if ((groups + u - 1) / u * u <= padded) { U = u; padded = (groups + u - 1) / u * u; }
+  const dim3 grid((unsigned)nrb, (unsigned)((groups + U - 1) / U));
+  constexpr int sm = grp_smem_bytes<double, 3, true>();
+  switch (U) {
+    case 1: spmm_grp_real64_kernel<1><<<grid, kThreads, sm, st>>>(a); break;
+    case 2: spmm_grp_real64_kernel<2><<<grid, kThreads, sm, st>>>(a); break;
+    case 3: spmm_grp_real64_kernel<3><<<grid, kThreads, sm, st>>>(a); break;
+    default: spmm_grp_real64_kernel<4><<<grid, kThreads, sm, st>>>(a); break;
+  }
 }
 
 template <typename R, int V, int G> static void grp_attrs_v() {
@@ -1765,8 +1804,11 @@ template <typename R, int G> static void grp_attrs() {
 void cocg_kernel_attrs() {
   static bool done = false;
   if (done) return;
-  cudaFuncSetAttribute(spmm_grp_real64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       grp_smem_bytes<double, 3, true>());
+  constexpr int sm64 = grp_smem_bytes<double, 3, true>();
+  cudaFuncSetAttribute(spmm_grp_real64_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
+  cudaFuncSetAttribute(spmm_grp_real64_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
+  cudaFuncSetAttribute(spmm_grp_real64_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
+  cudaFuncSetAttribute(spmm_grp_real64_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
   grp_attrs<float, 2>();
   grp_attrs<float, 3>();
   grp_attrs<float, 4>();
