@@ -214,6 +214,43 @@ __device__ __forceinline__ bool block_then_grid_reduce(double (&acc)[VEC][NQ], c
   return block_then_grid_reduce<VEC, NQ>(acc, W, w_tile0, rb, nrb, partial, counter, out, w_out, sm);
 }
 
+// Terms of the reduced sums.  FP64: one fused multiply-add per product (GB300 runs FP64 at 2
+// operations per clock and SM, and the update is bound by them): x^2, y^2 and x y of a residual
+// entry are summed apart and combined by sq_sums, 3 operations instead of 8, and a product of two
+// complex entries takes 4 instead of 6.  FP32 keeps its sums of whole terms.
+template <typename R> __device__ __forceinline__ void add_sq(R (&s)[3], cx_t<R> r) {
+  if constexpr (sizeof(R) == 8) {
+    s[0] = fma(r.x, r.x, s[0]);
+    s[1] = fma(r.x, r.y, s[1]);
+    s[2] = fma(r.y, r.y, s[2]);
+  } else {
+    s[0] += r.x * r.x - r.y * r.y;
+    s[1] += 2 * r.x * r.y;
+    s[2] += r.x * r.x + r.y * r.y;
+  }
+}
+// Re r^T r, Im r^T r and ||r||^2 of add_sq's sums.
+template <typename R> __device__ __forceinline__ void sq_sums(const R (&s)[3], double (&o)[3]) {
+  if constexpr (sizeof(R) == 8) {
+    o[0] = s[0] - s[2];
+    o[1] = 2 * s[1];
+    o[2] = s[0] + s[2];
+  } else {
+    o[0] = s[0];
+    o[1] = s[1];
+    o[2] = s[2];
+  }
+}
+template <typename R> __device__ __forceinline__ void add_prod(R (&s)[2], cx_t<R> p, cx_t<R> q) {
+  if constexpr (sizeof(R) == 8) {
+    s[0] = fma(-p.y, q.y, fma(p.x, q.x, s[0]));
+    s[1] = fma(p.y, q.x, fma(p.x, q.y, s[1]));
+  } else {
+    s[0] += p.x * q.x - p.y * q.y;
+    s[1] += p.x * q.y + p.y * q.x;
+  }
+}
+
 // ------------------------------------------------------------------------------ init
 // r0 = c g, p0 = r0, q0 = c (A g - sigma B g); reduce mu0 = p0^T q0, rho0 = r0^T r0, ||r0||^2.
 template <typename R, int V>
@@ -421,10 +458,7 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
           }
           rv.z[v] = cfms(al[v], qv.z[v], rv.z[v]);
         }
-        const C rr = rv.z[v];
-        acc[v][0] += rr.x * rr.x - rr.y * rr.y;
-        acc[v][1] += 2 * rr.x * rr.y;
-        acc[v][2] += rr.x * rr.x + rr.y * rr.y;
+        add_sq<R>(acc[v], rv.z[v]);
       }
       if (CHK(5, off + woff<V>(VEC - 1), (long long)a.n * a.W)) stv<R, VEC>(a.r + off, rv);
     }
@@ -518,9 +552,7 @@ __device__ __forceinline__ void cocg_update_body(const CocgArgs<R> &a, const int
   int w;
   double accd[VEC][NQ];
 #pragma unroll
-  for (int v = 0; v < VEC; ++v)
-#pragma unroll
-    for (int qq = 0; qq < NQ; ++qq) accd[v][qq] = (double)acc[v][qq];
+  for (int v = 0; v < VEC; ++v) sq_sums<R>(acc[v], accd[v]);
   if (!block_then_grid_reduce<VEC, NQ>(accd, a.W, w_tile0, rb, a.nrb, a.partial, a.counters + tile, out, w))
     return;
   if (threadIdx.x < 32 * VEC) {
@@ -694,8 +726,7 @@ __device__ __forceinline__ void cocg_spmm_body(const CocgArgs<R> &a, const int r
         const C qn = FRESH ? s : cfma(be, qv.z[v], s);
         pv.z[v] = pn;
         qv.z[v] = qn;
-        acc[v][0] += pn.x * qn.x - pn.y * qn.y;
-        acc[v][1] += pn.x * qn.y + pn.y * qn.x;
+        add_prod<R>(acc[v], pn, qn);
       }
       stv_cs<R, VEC>(a.p + off, pv);
       stv_cs<R, VEC>(a.q + off, qv);
@@ -994,8 +1025,7 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
             const C qn = FRESH ? sv : cfma(be[v], qv.z[v], sv);
             pv.z[v] = pn;
             qv.z[v] = qn;
-            acc[v][0] += pn.x * qn.x - pn.y * qn.y;
-            acc[v][1] += pn.x * qn.y + pn.y * qn.x;
+            add_prod<R>(acc[v], pn, qn);
           }
           stv_cs<R, VEC>(a.p + off, pv);
           stv_cs<R, VEC>(a.q + off, qv);
