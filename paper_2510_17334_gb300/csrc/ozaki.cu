@@ -9,13 +9,21 @@
 //
 // MMA kernel.  A work unit is a 128 x 32 output tile over a range of k-blocks; CTAs are
 // persistent (one per SM) and walk the units b, b + gridDim.x, ...:
-//   warp 4 lane 0   bulk-copies 7 A and 7 B slices per k-block into a 3-stage ring;
-//   warp 5          allocates TMEM; lane 0 issues 2 x 28 MMAs (M128 N32 K16) per k-block
-//                   into six accumulators (levels 0..4 and the merged 5..6) of one of two
+//   warp 8 lane 0   bulk-copies 7 A and 7 B slices per k-block into a 3-stage ring;
+//   warp 9          allocates TMEM; lane 0 issues 2 x 7 MMAs per k-block into seven
+//                   accumulators (levels 0..6, 32 columns each, side by side) of one of two
 //                   TMEM buffers, which alternate between 128-product chunks;
-//   warps 0-3       drain a finished buffer (tcgen05.ld, one TMEM lane quarter each) into
-//                   64-bit integer sums of the exact levels and an FP32 sum of the merged
-//                   level, while the next chunk runs on the other buffer.
+//   warps 0-7       drain a finished buffer (tcgen05.ld, one TMEM lane quarter and half of
+//                   the columns each) into 64-bit integer sums of the exact levels and an
+//                   FP32 sum of levels 5 and 6, while the next chunk runs on the other buffer.
+// The 7 B slices of a k-step lie one after the other in shared memory, so slice s of A times
+// the slices 0..6-s of B is one MMA of N = 32 (7 - s) whose columns are the levels s..6: every A
+// tile (4 KB) is read once per k-step instead of once per digit pair.  With 28 MMAs of N = 32,
+// 40 clocks of shared-memory reads each for 16 of math, the symmetric product of 68,921 x 160
+// blocks took 165 us, now 127 us.
+// The drain is a serial chain of conversions and 64-bit integer sums per warp (issue 19 % with
+// one drain warp per scheduler): with 8 drain warps instead of 4 Z = X S of 68,921 x 160 by
+// 160 x 160 went from 270 to 157 us.
 // Every wait is bounded by a 2 s deadline on the global timer; on expiry the CTA records a
 // code in *err, finishes its outstanding copies and MMAs, frees TMEM and returns.
 #include "ozaki.cuh"
@@ -26,8 +34,11 @@ namespace slrf {
 namespace {
 
 constexpr int kS = 7;          // digit slices
-constexpr int kAcc = 6;        // accumulators per TMEM buffer
+constexpr int kAcc = kS;       // accumulators per TMEM buffer: one per level
 constexpr int kTM = 128, kTN = 32;
+constexpr int kEpiWarps = 8;   // drain warps: a TMEM lane quarter and half of a level's columns each
+constexpr int kEN = kTN / 2;   // columns per drain warp
+constexpr int kOzThreads = 32 * (kEpiWarps + 2);
 constexpr int kChunkKB = 4;    // k-blocks (of 32) per exact chunk: 128 products
 constexpr int kStages = 3;
 constexpr int kATile = 4096;   // 128 rows x 16 products x 2 B
@@ -37,7 +48,7 @@ constexpr int kStageB = kS * 2 * kBTile;
 constexpr int kStage = kStageA + kStageB;
 constexpr int kBarOff = kStages * kStage;
 constexpr int kMmaSmem = kBarOff + 128;
-constexpr uint32_t kTmemCols = 512;  // 2 buffers x 6 accumulators x 32 columns = 384 used
+constexpr uint32_t kTmemCols = 512;  // 2 buffers x 7 accumulators x 32 columns = 448 used
 constexpr int kESent = (int)0x80808080;  // exponent of an all-zero row
 constexpr int kENonFinite = 4096;        // exponent marking a row with Inf/NaN
 constexpr int kMaxChunksPerCta = 64;     // keeps the 64-bit sums below 2^62
@@ -75,21 +86,19 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar))
                : "memory");
 }
-// 32 consecutive FP32 columns of this thread's TMEM lane; waits for the load.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
+// 16 consecutive FP32 columns of this thread's TMEM lane; waits for the load.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];\n"
       "tcgen05.wait::ld.sync.aligned;\n"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
 #pragma unroll
-  for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+  for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
 // Shared-memory descriptor, no swizzle, K-major: core matrices 128 B apart along K (LBO)
@@ -99,8 +108,9 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
          (1ull << 46);
 }
 // Instruction descriptor of kind::f16: FP32 accumulator, bf16 A and B, both K-major.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTN >> 3) << 17) |
-                            ((uint32_t)(kTM >> 4) << 24);
+constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
+}
 
 // ------------------------------------------------------------------------- splitting
 __device__ __forceinline__ int exp_of(double x) {  // E with |x| < 2^E (0 / subnormal: sentinel)
@@ -233,6 +243,30 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(int64_t n, const dou
   }
 }
 
+// Bits of the FP64 value (I 2^-32 + f) 2^(e + 32) with the exact levels I and the FP32 sum f of
+// the others (|f| < 2^-14, |I| < 2^58 for up to 512 products): I is shifted up by as many bits as
+// it has to spare (at most 12), f added in those units -- finer than the result's last place --
+// and the sum rounded to 53 bits, all in integers.  GB300 runs FP64 at 2 operations per clock and
+// SM, and three operations an output (11 million of them in a 68,921 x 160 block) would take
+// 57 us of it.
+__device__ __forceinline__ long long finish(long long I, float f, int e) {
+  const unsigned long long a0 = (unsigned long long)(I < 0 ? -I : I);
+  const int sh = min(max(__clzll((long long)a0) - 2, 0), 12);
+  const long long v = (I << sh) + (long long)__float2int_rn(f * __int_as_float((127 + 32 + sh) << 23));
+  if (v == 0) return 0;
+  const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << lz;  // leading one in bit 63
+  unsigned long long q = m >> 11;
+  const unsigned rem = (unsigned)m & 0x7FFu;
+  q += (rem > 0x400u || (rem == 0x400u && (q & 1))) ? 1u : 0u;
+  const int ex = 1023 + 63 - lz + e - sh;
+  const long long sign = v & (long long)0x8000000000000000ull;
+  if (ex < 1 || ex > 2045)  // subnormal or beyond range
+    return __double_as_longlong(scalbn((double)v, e - sh));
+  return sign | (long long)(((unsigned long long)(ex - 1) << 52) + q);
+}
+
 // ------------------------------------------------------------------------- MMA kernel
 struct OzMma {
   const uint16_t *dA, *dB;
@@ -249,6 +283,7 @@ struct OzMma {
   int ldz;
   int64_t rows;
   int cols;
+  int zpairs;  // rows of Z start on 16-byte boundaries: two columns per access
   double alpha, beta;
   int *err;
   const int *run_if;
@@ -278,7 +313,7 @@ __device__ __forceinline__ void unit_of(const OzMma &p, int q, int &t, int &u, i
 // Persistent: CTA b takes the units b, b + gridDim.x, ...; the three roles walk the same
 // sequence, so the copy ring, the MMA stream and the TMEM double buffer run on across
 // unit boundaries (k-block counter g, chunk counter c).
-__global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
+__global__ void __launch_bounds__(kOzThreads, 1) oz_mma_kernel(const OzMma p) {
   if (p.run_if != nullptr && *p.run_if == 0) return;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kBarOff);
@@ -287,17 +322,17 @@ __global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull + b, 1); mbar_init(tempty + b, 128); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull + b, 1); mbar_init(tempty + b, 32 * kEpiWarps); }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 5) tmem_alloc(tslot, kTmemCols);
+  if (warp == kEpiWarps + 1) tmem_alloc(tslot, kTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
 
-  if (warp == 4) {
+  if (warp == kEpiWarps) {
     if (lane == 0) {
       int g = 0;
       bool ok = true;
@@ -316,7 +351,7 @@ __global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
             for (int j = 0; j < 2; ++j) {
               bulk_g2s(sa + (sl * 2 + j) * kATile, p.dA + off16(sl, p.KB, kb, j, p.RA8, 16 * t, 0, 0) * 8, kATile,
                        full + s_);
-              bulk_g2s(sb + (sl * 2 + j) * kBTile, p.dB + off16(sl, p.KB, kb, j, p.RB8, 4 * u, 0, 0) * 8, kBTile,
+              bulk_g2s(sb + (j * kS + sl) * kBTile, p.dB + off16(sl, p.KB, kb, j, p.RB8, 4 * u, 0, 0) * 8, kBTile,
                        full + s_);
             }
         }
@@ -324,7 +359,7 @@ __global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
       // every armed stage has landed before the CTA may exit (a no-op in normal runs)
       for (int i = max(0, g - kStages); i < g; ++i) mbar_wait(full + i % kStages, (i / kStages) & 1, p.err, 6);
     }
-  } else if (warp == 5) {
+  } else if (warp == kEpiWarps + 1) {
     if (lane == 0) {
       const uint32_t sbase = su32(smem);
       int g = 0, c = 0, buf = 0;
@@ -346,14 +381,9 @@ __global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
 #pragma unroll
           for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int sl = 0; sl < kS; ++sl)
-#pragma unroll
-              for (int tl = 0; tl + sl < kS; ++tl) {
-                const int lvl = sl + tl < 5 ? sl + tl : 5;
-                const uint32_t acc = (first && j == 0 && sl == 0 && tl <= 5) ? 0u : 1u;
-                mma_bf16(dbuf + (uint32_t)(lvl * kTN), sdesc(a0 + (sl * 2 + j) * kATile),
-                         sdesc(b0 + (tl * 2 + j) * kBTile), kIdesc, acc);
-              }
+            for (int sl = 0; sl < kS; ++sl)  // slice 0 covers every level: it starts the chunk's sums
+              mma_bf16(dbuf + (uint32_t)(sl * kTN), sdesc(a0 + (sl * 2 + j) * kATile), sdesc(b0 + j * kS * kBTile),
+                       idesc(kTN * (kS - sl)), (first && j == 0 && sl == 0) ? 0u : 1u);
           mma_commit(empty + s_);
           if ((i % kChunkKB) == kChunkKB - 1 || i == nkb - 1) {
             mma_commit(tfull + buf);
@@ -366,81 +396,99 @@ __global__ void __launch_bounds__(192, 1) oz_mma_kernel(const OzMma p) {
     }
     __syncwarp();
   } else {
-    // epilogue: warp w owns TMEM lanes 32w..32w+31 = output rows 128t + 32w + lane
+    // epilogue: warps q and q + 4 own TMEM lanes 32q..32q+31 = output rows 128t + 32q + lane,
+    // the first the columns 0..15 of the tile, the other 16..31
+    const int quarter = warp & 3, n0 = (warp >> 2) * kEN;
     int c = 0;
     bool ok = true;
     for (int q = blockIdx.x; q < p.units && ok; q += gridDim.x) {
       int t, u, split, kb0, nkb;
       unit_of(p, q, t, u, split, kb0, nkb);
-      long long I[32];
-      float f5[32];
+      long long I[kEN];
+      float f5[kEN];
 #pragma unroll
-      for (int qq = 0; qq < 32; ++qq) { I[qq] = 0; f5[qq] = 0.f; }
+      for (int qq = 0; qq < kEN; ++qq) { I[qq] = 0; f5[qq] = 0.f; }
       const int nch = (nkb + kChunkKB - 1) / kChunkKB;
       for (int k = 0; k < nch; ++k, ++c) {
         const int buf = c & 1;
         if (!mbar_wait(tfull + buf, (c >> 1) & 1, p.err, 5)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tb = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(buf * kAcc * kTN);
-        float v[32];
+        const uint32_t tb = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(buf * kAcc * kTN + n0);
+        float v[kEN];
 #pragma unroll
         for (int lvl = 0; lvl < 5; ++lvl) {
-          tmem_ld32(tb + (uint32_t)(lvl * kTN), v);
+          tmem_ld16(tb + (uint32_t)(lvl * kTN), v);
           const float sc = __int_as_float((127 + 8 * lvl) << 23);  // 2^(8 lvl)
 #pragma unroll
-          for (int qq = 0; qq < 32; ++qq)
+          for (int qq = 0; qq < kEN; ++qq)
             I[qq] += (long long)__float2int_rn(v[qq] * sc) * (1ll << (8 * (4 - lvl)));
         }
-        tmem_ld32(tb + (uint32_t)(5 * kTN), v);
 #pragma unroll
-        for (int qq = 0; qq < 32; ++qq) f5[qq] += v[qq];
+        for (int lvl = 5; lvl < kS; ++lvl) {
+          tmem_ld16(tb + (uint32_t)(lvl * kTN), v);
+#pragma unroll
+          for (int qq = 0; qq < kEN; ++qq) f5[qq] += v[qq];
+        }
         tc_fence_before();
         mbar_arrive(tempty + buf);
       }
       if (!ok) break;
-      // Sum of the levels in FP64 (the merged levels keep their FP32 sum's bits: rounding
-      // them into the 64-bit units would cost 2^-49 of a single product); powers of two are
-      // applied to the exponent bits.  GB300 runs FP64 at 2 operations per clock per SM, so
-      // the finish of 128 x 32 outputs per unit is kept to three FP64 operations each.
-      const int64_t row = (int64_t)kTM * t + 32 * warp + lane;
+      // Sum of the levels: in FP64 for the partial tiles of a Gram product, in integers for the
+      // outputs of a projection (finish), which are many.
+      const int64_t row = (int64_t)kTM * t + 32 * quarter + lane;
+      const int col0 = kTN * u + n0;
       if (p.mode == 0) {
-        double *dst = p.part + ((int64_t)split * p.MR + row) * p.NC + kTN * u;
+        double2 *dst = reinterpret_cast<double2 *>(p.part + ((int64_t)split * p.MR + row) * p.NC + col0);
 #pragma unroll
-        for (int qq = 0; qq < 32; ++qq) dst[qq] = fma((double)I[qq], 0x1p-32, (double)f5[qq]);
+        for (int qq = 0; qq < kEN; qq += 2)
+          dst[qq / 2] = make_double2(fma((double)I[qq], 0x1p-32, (double)f5[qq]),
+                                     fma((double)I[qq + 1], 0x1p-32, (double)f5[qq + 1]));
       } else if (row < p.rows) {
         const int ea = max(p.EA[row], -1100);
         // uniform flags, decided once (FP64 compares run on the FP64 pipe)
         const int amode = p.alpha == 1.0 ? 0 : (p.alpha == -1.0 ? 1 : 2);
         const int bmode = p.beta == 0.0 ? 0 : (p.beta == 1.0 ? 1 : 2);
-#pragma unroll
-        for (int qq = 0; qq < 32; ++qq) {
-          const int col = kTN * u + qq;
-          if (col >= p.cols) continue;
-          const int eb = max(p.EB[col], -1100);
-          double z = fma((double)f5[qq], 4294967296.0, (double)I[qq]);  // in units of 2^-32
-          const int e = ea + eb - 48;  // value = z 2^(EA + EB - 16 - 32)
-          long long zb = __double_as_longlong(z);
-          if (ea == kENonFinite || eb == kENonFinite) {
-            zb = 0x7ff8000000000000ll;
-          } else if ((zb & 0x7FFFFFFFFFFFFFFFll) != 0) {
-            const int ez = (int)((zb >> 52) & 0x7FF);  // biased exponent of z (>= 1023)
-            if (ez + e >= 1 && ez + e <= 2046) zb += (long long)e << 52;
-            else zb = __double_as_longlong(scalbn(z, e));
-          }
+        double *const zrow = p.Z + row * p.ldz + col0;
+        // alpha times the product, column col0 + qq
+        auto value = [&](int qq) -> double {
+          const int eb = max(p.EB[col0 + qq], -1100);
+          long long zb = finish(I[qq], f5[qq], ea + eb - 48);
+          if (ea == kENonFinite || eb == kENonFinite) zb = 0x7ff8000000000000ll;
           if (amode == 1) zb ^= (long long)0x8000000000000000ull;  // alpha = -1: flip the sign bit
-          z = __longlong_as_double(zb);
-          if (amode == 2) z *= p.alpha;
-          double *zp = p.Z + row * p.ldz + col;
-          if (bmode == 1) z += *zp;
-          else if (bmode == 2) z = fma(p.beta, *zp, z);
-          *zp = z;
+          const double z = __longlong_as_double(zb);
+          return amode == 2 ? z * p.alpha : z;
+        };
+        auto plus = [&](double z, double o) { return bmode == 1 ? z + o : fma(p.beta, o, z); };
+        if (p.zpairs && col0 + kEN <= p.cols) {
+          double2 *const zp = reinterpret_cast<double2 *>(zrow);
+#pragma unroll
+          for (int h = 0; h < kEN / 8; ++h) {  // old values four at a time, ahead of their use
+            double2 o[4];
+            if (bmode != 0) {
+#pragma unroll
+              for (int w = 0; w < 4; ++w) o[w] = zp[4 * h + w];
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              double2 z = make_double2(value(8 * h + 2 * w), value(8 * h + 2 * w + 1));
+              if (bmode != 0) z = make_double2(plus(z.x, o[w].x), plus(z.y, o[w].y));
+              zp[4 * h + w] = z;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int qq = 0; qq < kEN; ++qq)
+            if (col0 + qq < p.cols) {
+              const double z = value(qq);
+              zrow[qq] = bmode != 0 ? plus(z, zrow[qq]) : z;
+            }
         }
       }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) {
+  if (warp == kEpiWarps + 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
@@ -591,7 +639,7 @@ void oz_gram(int64_t n, const double *X, int ldx, int k1, const double *Y, int l
   p.run_if = run_if;
   p.tiles = g.tiles;
   p.units = g.tiles * g.nsplit;
-  oz_mma_kernel<<<std::min(p.units, num_sms()), 192, kMmaSmem, st>>>(p);
+  oz_mma_kernel<<<std::min(p.units, num_sms()), kOzThreads, kMmaSmem, st>>>(p);
   const int64_t tot = (int64_t)k1 * k2;
   oz_gram_finalize_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(k1, k2, g.nsplit, g.MR, g.NC, part, EA, EB,
                                                                         sym ? 1 : 0, C, ldc, run_if);
@@ -635,10 +683,11 @@ void oz_gemm(int64_t n, const double *X, int ldx, int k1, const double *S, int l
   p.EA = EA; p.EB = EB;
   p.Z = Z; p.ldz = ldz; p.rows = n; p.cols = k2;
   p.alpha = alpha; p.beta = beta;
+  p.zpairs = ldz % 2 == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0;
   p.err = err;
   p.tiles = p.m_tiles * p.n_tiles;
   p.units = p.tiles;
-  oz_mma_kernel<<<std::min(p.units, num_sms()), 192, kMmaSmem, st>>>(p);
+  oz_mma_kernel<<<std::min(p.units, num_sms()), kOzThreads, kMmaSmem, st>>>(p);
 }
 
 }  // namespace slrf

@@ -10,7 +10,7 @@
 //
 // Exactness.  The products D_s E_t of level l = s + t are integers times 2^(-8l); summed over
 // 128 rows (one chunk) every level l <= 4 stays below 2^24 units, so the FP32 tensor-core
-// accumulation of each such level is exact.  Levels 5 and 6 share one accumulator (their
+// accumulation of each such level is exact.  Levels 5 and 6 are summed in FP32 (their
 // weight is below 2^-40 of the leading term); levels above 6 are dropped (below 2^-56).
 // Chunk results of the exact levels are combined in 64-bit integers, so the per-block sums
 // are exact and deterministic; blocks of rows are summed in FP64 in a fixed order.
