@@ -76,21 +76,29 @@ __global__ void __launch_bounds__(256) spmm_real_kernel(int64_t n, const int64_t
   }
 }
 
-// YB = B X with FP32 products and sums (FP64 in and out): for the first Cholesky-QR pass,
-// whose Gram matrix is formed in FP32 anyway.  Same work split as spmm_real_kernel; the
-// CSR chunk reaches the lanes by two 32-bit shuffles per entry.
+// YB = B X with FP32 products and sums: for the first Cholesky-QR pass, whose Gram matrix is
+// formed in FP32 anyway.  Same work split as spmm_real_kernel; the CSR chunk reaches the lanes
+// by two 32-bit shuffles per entry.  X32 is the FP32 copy of X (to_f32_kernel): GB300 converts
+// FP64 on its FP64 pipe, and converting every gathered value (27 times each) took as long as an
+// FP64 product: 68,921 rows, 160 columns 0.49 -> 0.11 ms.
+__global__ void __launch_bounds__(256) to_f32_kernel(int64_t n, int k, const double *__restrict__ X, int ldx,
+                                                     float *__restrict__ Y) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n * k) return;
+  Y[t] = (float)X[t / k * ldx + t % k];
+}
 template <int U>
 __global__ void __launch_bounds__(256) spmm_b32_kernel(int64_t n, const int64_t *__restrict__ rowptr,
                                                        const int32_t *__restrict__ col,
                                                        const double *__restrict__ valB,
-                                                       const double *__restrict__ X, int ldx, int k,
+                                                       const float *__restrict__ X32, int k,
                                                        double *__restrict__ YB, int ldy) {
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * kSpmmRows + (threadIdx.x >> 5);
   if (i >= n) return;
   const int c0 = blockIdx.y * (32 * U) + lane;
-  const char *const xl = reinterpret_cast<const char *>(X + c0);
-  const unsigned row_bytes = (unsigned)ldx * (unsigned)sizeof(double);
+  const char *const xl = reinterpret_cast<const char *>(X32 + c0);
+  const unsigned row_bytes = (unsigned)k * (unsigned)sizeof(float);
   float sb[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) sb[u] = 0.f;
@@ -107,10 +115,10 @@ __global__ void __launch_bounds__(256) spmm_b32_kernel(int64_t n, const int64_t 
     for (int t = 0; t < cnt; ++t) {
       const int c = __shfl_sync(0xffffffffu, cl, t);
       const float b = __shfl_sync(0xffffffffu, bl, t);
-      const double *xr = reinterpret_cast<const double *>(xl + (unsigned long long)(unsigned)c * row_bytes);
+      const float *xr = reinterpret_cast<const float *>(xl + (unsigned long long)(unsigned)c * row_bytes);
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (c0 + 32 * u < k) sb[u] = fmaf(b, (float)xr[32 * u], sb[u]);
+        if (c0 + 32 * u < k) sb[u] = fmaf(b, xr[32 * u], sb[u]);
     }
   }
 #pragma unroll
@@ -306,11 +314,13 @@ void spmm_real(int64_t n, const int64_t *rowptr, const int32_t *col, const doubl
 }
 
 void spmm_b32(int64_t n, const int64_t *rowptr, const int32_t *col, const double *valB, const double *X, int ldx,
-              int k, double *YB, int ldy, cudaStream_t st) {
+              int k, float *x32, double *YB, int ldy, cudaStream_t st) {
   if (n <= 0 || k <= 0) return;
+  const int64_t tot = n * k;
+  to_f32_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n, k, X, ldx, x32);
   const int U = spmm_lanes(k);
   dim3 grid((unsigned)((n + kSpmmRows - 1) / kSpmmRows), (unsigned)((k + 32 * U - 1) / (32 * U)));
-#define SPMM_B32(UU) spmm_b32_kernel<UU><<<grid, 256, 0, st>>>(n, rowptr, col, valB, X, ldx, k, YB, ldy)
+#define SPMM_B32(UU) spmm_b32_kernel<UU><<<grid, 256, 0, st>>>(n, rowptr, col, valB, x32, k, YB, ldy)
   switch (U) {
     case 1: SPMM_B32(1); break;
     case 2: SPMM_B32(2); break;
@@ -416,36 +426,51 @@ __global__ void __launch_bounds__(256) gram_partial_kernel(int64_t n, const doub
     }
 }
 
-// The same product with FP32 inputs and FP32 accumulation inside each row chunk (chunk
-// partials are summed in FP64): a Gram accurate to ~1e-6 relative, used where a later
-// FP64 pass removes its error (first Cholesky-QR pass, first CGS pass).
-__global__ void __launch_bounds__(256) gram32_partial_kernel(int64_t n, const double *__restrict__ X, int ldx, int k1,
-                                                             const double *__restrict__ Y, int ldy, int k2,
+// The same product from FP32 copies of X (n x k1) and Y (n x k2) with FP32 accumulation inside
+// each row chunk (chunk partials are summed in FP64): a Gram accurate to ~1e-6 relative, used
+// where a later FP64 pass removes its error (first Cholesky-QR pass, first CGS pass).  The
+// copies come first because every value is read by several tiles and GB300 converts FP64 on its
+// FP64 pipe; the next rows load while the current ones are multiplied.  68,921 rows, 160 x 160:
+// 0.38 ms converting in place -> 0.26 ms with the copies.
+__global__ void __launch_bounds__(256) gram32_partial_kernel(int64_t n, const float *__restrict__ X, int k1,
+                                                             const float *__restrict__ Y, int k2,
                                                              int64_t rows_per_chunk, bool sym,
                                                              double *__restrict__ work, const int *run_if) {
   if (run_if != nullptr && *run_if == 0) return;
   const int ti = blockIdx.x, tj = blockIdx.y, z = blockIdx.z;
   if (sym && ti > tj) return;
-  __shared__ float xs[kGR][kGT];
-  __shared__ float ys[kGR][kGT];
+  __shared__ __align__(16) float xs[kGR][kGT];
+  __shared__ __align__(16) float ys[kGR][kGT];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int lc = threadIdx.x & (kGT - 1), lr = threadIdx.x >> 6;  // this thread's column and first row of a load
+  const int cx = ti * kGT + lc, cy = tj * kGT + lc;
   float acc[4][4] = {};
   const int64_t r0 = (int64_t)z * rows_per_chunk;
   const int64_t r1 = (r0 + rows_per_chunk < n) ? r0 + rows_per_chunk : n;
+  constexpr int NL = kGR / 4;  // rows per thread and load
+  float nx[NL], ny[NL];
+  auto load = [&](int64_t rr) {
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+      const int64_t row = rr + lr + 4 * u;
+      nx[u] = (row < r1 && cx < k1) ? X[row * k1 + cx] : 0.0f;
+      ny[u] = (row < r1 && cy < k2) ? Y[row * k2 + cy] : 0.0f;
+    }
+  };
+  load(r0);
   for (int64_t rr = r0; rr < r1; rr += kGR) {
-    for (int t = threadIdx.x; t < kGR * kGT; t += 256) {
-      const int lr = t / kGT, lc = t % kGT;
-      const int64_t row = rr + lr;
-      const int cx = ti * kGT + lc, cy = tj * kGT + lc;
-      xs[lr][lc] = (row < r1 && cx < k1) ? (float)X[row * ldx + cx] : 0.0f;
-      ys[lr][lc] = (row < r1 && cy < k2) ? (float)Y[row * ldy + cy] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+      xs[lr + 4 * u][lc] = nx[u];
+      ys[lr + 4 * u][lc] = ny[u];
     }
     __syncthreads();
+    if (rr + kGR < r1) load(rr + kGR);
 #pragma unroll
-    for (int lr = 0; lr < kGR; ++lr) {
-      float a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { a[u] = xs[lr][ty * 4 + u]; b[u] = ys[lr][tx * 4 + u]; }
+    for (int l = 0; l < kGR; ++l) {
+      const float4 av = *reinterpret_cast<const float4 *>(&xs[l][ty * 4]);
+      const float4 bv = *reinterpret_cast<const float4 *>(&ys[l][tx * 4]);
+      const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -478,8 +503,8 @@ __global__ void gram_reduce_kernel(int k1, int k2, int nz, bool sym, const doubl
 
 static int gram_chunks(int64_t n, int k1, int k2) {
   const int tiles = ((k1 + kGT - 1) / kGT) * ((k2 + kGT - 1) / kGT);
-  int nz = (2 * device_sm_count() + tiles - 1) / tiles;
-  const int64_t maxz = (n + 255) / 256;
+  int nz = (4 * device_sm_count() + tiles - 1) / tiles;
+  const int64_t maxz = (n + 63) / 64;
   if (nz > maxz) nz = (int)maxz;
   if (nz < 1) nz = 1;
   if (nz > 64) nz = 64;
@@ -489,13 +514,17 @@ static int gram_chunks(int64_t n, int k1, int k2) {
 size_t gram_work_doubles(int64_t n, int k1, int k2) { return (size_t)gram_chunks(n, k1, k2) * k1 * k2; }
 
 void gram(int64_t n, const double *X, int ldx, int k1, const double *Y, int ldy, int k2, double *C, int ldc,
-          bool sym, double *work, cudaStream_t st, bool fp32, const int *run_if) {
+          bool sym, double *work, cudaStream_t st, float *f32, const int *run_if) {
   if (k1 <= 0 || k2 <= 0) return;
   const int nz = gram_chunks(n, k1, k2);
   const int64_t rpc = (n + nz - 1) / nz;
   dim3 grid((k1 + kGT - 1) / kGT, (k2 + kGT - 1) / kGT, nz);
-  if (fp32) gram32_partial_kernel<<<grid, 256, 0, st>>>(n, X, ldx, k1, Y, ldy, k2, rpc, sym, work, run_if);
-  else gram_partial_kernel<<<grid, 256, 0, st>>>(n, X, ldx, k1, Y, ldy, k2, rpc, sym, work, run_if);
+  if (f32 != nullptr) {
+    float *const x = f32, *const y = f32 + (size_t)n * k1;
+    to_f32_kernel<<<(unsigned)((n * k1 + 255) / 256), 256, 0, st>>>(n, k1, X, ldx, x);
+    to_f32_kernel<<<(unsigned)((n * k2 + 255) / 256), 256, 0, st>>>(n, k2, Y, ldy, y);
+    gram32_partial_kernel<<<grid, 256, 0, st>>>(n, x, k1, y, k2, rpc, sym, work, run_if);
+  } else gram_partial_kernel<<<grid, 256, 0, st>>>(n, X, ldx, k1, Y, ldy, k2, rpc, sym, work, run_if);
   const int64_t tot = (int64_t)k1 * k2;
   gram_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(k1, k2, nz, sym, work, C, ldc, run_if);
 }
@@ -730,24 +759,29 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int l
     D[i][l] = (i < b && l <= i) ? G[(size_t)(j0 + i) * ldg + j0 + l] : 0.0;
   }
   __syncthreads();
-  // unblocked right-looking factorisation of D by warp 0 (lane i owns row i)
-  if (tid < 32) {
-    const int i = tid;
-    for (int j = 0; j < b; ++j) {
-      if (i == j) {
-        const double d = D[j][j];
-        if (!(d > 0.0) || !isfinite(d)) fail = 1;
-        D[j][j] = (d > 0.0 && isfinite(d)) ? sqrt(d) : 1.0;
+  // Right-looking factorisation of D.  A warp's FP64 operation takes 16 clocks of the SM, so a
+  // column's reciprocal root is taken by one warp and there is no division, the trailing update
+  // is spread over the rows' warps, and so are the panel rows below.  With one warp for each (a
+  // division per row and column) a panel launch took 64 us; now 23 us.
+  __shared__ double inv[kCb];  // 1 / L[j][j]
+  for (int j = 0; j < b; ++j) {
+    if (tid < 32) {
+      const double d = D[j][j];
+      const bool ok = d > 0.0 && isfinite(d);
+      const double r = ok ? rsqrt(d) : 1.0;
+      __syncwarp();
+      if (tid >= j) D[tid][j] = tid == j ? (ok ? d * r : 1.0) : D[tid][j] * r;
+      if (tid == j) {
+        inv[j] = r;
+        if (!ok) fail = 1;
       }
-      __syncwarp();
-      if (i > j && i < b) D[i][j] /= D[j][j];
-      __syncwarp();
-      if (i > j && i < b)
-        for (int l = j + 1; l <= i; ++l) D[i][l] -= D[i][j] * D[l][j];
-      __syncwarp();
     }
+    __syncthreads();
+    const int l = tid & 31;
+    for (int i = j + 1 + (tid >> 5); i < b; i += 8)
+      if (l > j && l <= i) D[i][l] = fma(-D[i][j], D[l][j], D[i][l]);
+    __syncthreads();
   }
-  __syncthreads();
   if (fail) {
     if (blockIdx.x == 0 && tid == 0) atomicExch(status, SLRF_ECHOL);
     return;
@@ -757,26 +791,44 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int l
       const int i = e / b, l = e % b;
       if (l <= i) G[(size_t)(j0 + i) * ldg + j0 + l] = D[i][l];
     }
-  // panel rows of this CTA: forward substitution with D^T, one row per thread
-  const int j1 = j0 + b;
-  const int r = j1 + (int)blockIdx.x * kCb + tid;
-  if (tid < kCb && r < k) {
-    double x[kCb];
-    double *row = G + (size_t)r * ldg + j0;
+  // panel rows of this CTA: forward substitution with D^T, column by column; thread (row, part)
+  // of the first four warps keeps the columns part, part + 4, ...
+  const int r0 = j0 + b + (int)blockIdx.x * kCb, nr = min(kCb, k - r0);
+  if (nr <= 0) return;
+  __shared__ double P[kCb][kCb + 1];
+  for (int e = tid; e < kCb * kCb; e += blockDim.x) {
+    const int rr = e / kCb, c = e % kCb;
+    P[rr][c] = (rr < nr && c < b) ? G[(size_t)(r0 + rr) * ldg + j0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int row = tid & 31, part = tid >> 5;
+  double x[kCb / 4];
+  if (part < 4) {
 #pragma unroll
-    for (int c = 0; c < kCb; ++c) x[c] = c < b ? row[c] : 0.0;
+    for (int u = 0; u < kCb / 4; ++u) x[u] = P[row][part + 4 * u];
+  }
 #pragma unroll
-    for (int c = 0; c < kCb; ++c) {
-      if (c < b) {
-        double v = x[c];
+  for (int q = 0; q < kCb / 4; ++q) {
 #pragma unroll
-        for (int l = 0; l < c; ++l) v -= x[l] * D[c][l];
-        x[c] = v / D[c][c];
+    for (int s = 0; s < 4; ++s) {
+      const int c = 4 * q + s;
+      if (c >= b) break;
+      if (part == s) {
+        x[q] *= inv[c];
+        P[row][c] = x[q];
+      }
+      __syncthreads();
+      if (part < 4) {
+        const double xc = P[row][c];
+        if (part > s) x[q] = fma(-xc, D[part + 4 * q][c], x[q]);
+#pragma unroll
+        for (int u = q + 1; u < kCb / 4; ++u) x[u] = fma(-xc, D[part + 4 * u][c], x[u]);
       }
     }
-#pragma unroll
-    for (int c = 0; c < kCb; ++c)
-      if (c < b) row[c] = x[c];
+  }
+  for (int e = tid; e < kCb * kCb; e += blockDim.x) {
+    const int rr = e / kCb, c = e % kCb;
+    if (rr < nr && c < b) G[(size_t)(r0 + rr) * ldg + j0 + c] = P[rr][c];
   }
 }
 __global__ void __launch_bounds__(256) chol_syrk_kernel(int k, double *G, int ldg, int j0, int b, int *status,
@@ -824,6 +876,7 @@ __global__ void __launch_bounds__(256) tri_inv_kernel(int k, const double *G, in
   constexpr int kParts = 256 / (kCi * kCi);
   __shared__ double S[kParts][kCi][kCi];
   __shared__ double Ld[kCi][kCi + 1];  // the row block's diagonal block of L
+  __shared__ double Li[kCi];           // 1 / its diagonal
   for (int i0 = c0; i0 < k; i0 += kCi) {
     const int bi = min(kCi, k - i0);
     // S = L[I][c0 .. i0) X[c0 .. i0)[C]  (independent loads: several in flight per thread)
@@ -840,17 +893,23 @@ __global__ void __launch_bounds__(256) tri_inv_kernel(int k, const double *G, in
       Ld[a][b] = (a < bi && b <= a) ? G[(size_t)(i0 + a) * ldg + i0 + b] : 0.0;
     }
     __syncthreads();
-    // forward substitution inside the block (one thread per column)
-    if (tid < kCi) {
-      const int c = tid, col = c0 + c;
-      for (int rr = 0; rr < bi; ++rr) {
-        const int row = i0 + rr;
-        double v = row == col ? 1.0 : 0.0;
+    if (tid < kCi) Li[tid] = tid < bi ? 1.0 / Ld[tid][tid] : 1.0;
+    __syncthreads();
+    // forward substitution inside the block: thread (row, column), a column in 8 lanes, row l's
+    // value to the others by a shuffle (with one thread per column and a division per row this
+    // chain was most of the launch: k = 160 104 us, now 50 us)
+    if (tid < kCi * kCi) {
+      const int rr = tid % kCi, c = tid / kCi, lane = tid & 31;
+      double v = i0 + rr == c0 + c ? 1.0 : 0.0;
 #pragma unroll
-        for (int q = 0; q < kParts; ++q) v -= S[q][rr][c];
-        for (int l = 0; l < rr; ++l) v -= Ld[rr][l] * X[(size_t)(i0 + l) * kCi + c];
-        X[(size_t)row * kCi + c] = row < col ? 0.0 : v / Ld[rr][rr];
+      for (int q = 0; q < kParts; ++q) v -= S[q][rr][c];
+#pragma unroll
+      for (int l = 0; l < kCi; ++l) {
+        if (rr == l) v *= Li[l];
+        const double xl = __shfl_sync(0xffffffffu, v, (lane & ~(kCi - 1)) + l);
+        if (rr > l) v = fma(-Ld[rr][l], xl, v);
       }
+      if (rr < bi) X[(size_t)(i0 + rr) * kCi + c] = i0 + rr < c0 + c ? 0.0 : v;
     }
     __syncthreads();
   }
@@ -908,8 +967,9 @@ void chol_inv(int k, double *G, int ldg, double *Rinv, int ldr, int *status, cud
 // round, but from a small table that the owners of the previous round filled (two copies,
 // alternating by round), and the block's own rows load together with them: a round costs
 // one L2 round trip, the rotation arithmetic and the barrier.  The sweep loop stops once
-// every off-diagonal met in a sweep is below 1e-8 of its diagonal scale (quadratic
-// convergence leaves them at rounding level after that sweep).
+// every off-diagonal met in a sweep is below 1e-9 of its diagonal scale (quadratic
+// convergence leaves them at rounding level after that sweep; at 1e-8 the clusters of a cube's
+// spectrum were left at up to 5e-9 of it).
 __device__ __forceinline__ void rr_pair(int kk, int r, int b, int &p, int &q) {
   const int M = kk - 1;
   int a0, a1;
@@ -929,18 +989,37 @@ __device__ __forceinline__ int rr_partner(int kk, int r, int x) {
 // t^2 + 2 tau t - 1 = 0 with tau = (a_qq - a_pp) / (2 a_pq), written as
 // t = sgn(th) ph / (|th| + sqrt(th^2 + ph^2)) with th = a_qq - a_pp, ph = 2 a_pq
 // (t = 1 when th = 0), then c = 1 / sqrt(1 + t^2), s = t c.
+// Every block computes every rotation of a round, so a round's FP64 time is mostly this
+// function's.  t is taken in FP32 (th and ph scaled so that the larger one is in [1, 2)): a
+// rotation is orthogonal whatever its angle, it only leaves 1e-7 of the entry it annihilates
+// (which is therefore not set to zero), and the next sweep meets that remainder.  c is refined
+// from FP32 by two Newton steps on c^-2 = 1 + t^2, so c^2 + s^2 = 1 to rounding: 15 FP64
+// operations, against 60 with an FP64 square root, division and reciprocal root.
+__device__ __forceinline__ int exp_bits(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
+__device__ __forceinline__ float scale_f(double x, int e) {  // x 2^e; 0 for 0, subnormals and underflow
+  const long long b = __double_as_longlong(x);
+  const int e0 = (int)((b >> 52) & 0x7FF), ex = e0 + e;
+  return e0 == 0 || ex <= 0 ? 0.f
+                            : (float)__longlong_as_double((b & ~(0x7FFll << 52)) | ((long long)ex << 52));
+}
 __device__ __forceinline__ void jacobi_rotation(double app, double aqq, double apq, double &c, double &sn) {
-  const double th = aqq - app, ph = 2.0 * apq;
-  double t;
-  if (fmax(fabs(th), fabs(ph)) < 1e150) {
-    const double num = th > 0.0 ? ph : (th < 0.0 ? -ph : fabs(ph));
-    t = num / (fabs(th) + sqrt(th * th + ph * ph));
-  } else {  // squares would overflow
-    const double tau = th / ph;
-    t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+  const double th = aqq - app, ph = apq + apq;
+  const int em = max(exp_bits(th), exp_bits(ph));
+  if (em >= 0x7FF) {  // not finite
+    c = 1.0;
+    sn = 0.0;
+    return;
   }
-  c = rsqrt(1.0 + t * t);
-  sn = t * c;
+  const float tf = scale_f(th, 1023 - em), pf = scale_f(ph, 1023 - em);
+  const float at = fabsf(tf);
+  float t = __fdividef(pf, at + sqrtf(fmaf(tf, tf, pf * pf)));
+  t = tf > 0.f ? t : (tf < 0.f ? -t : fabsf(t));  // th = 0: t = 1
+  const double td = (double)t, q = fma(td, td, 1.0);
+  double r = (double)rsqrtf(fmaf(t, t, 1.f));
+  r = fma(r * 0.5, fma(-q * r, r, 1.0), r);
+  r = fma(r * 0.5, fma(-q * r, r, 1.0), r);
+  c = r;
+  sn = td * r;
 }
 
 constexpr int kJacobiThreads = 128;
@@ -971,7 +1050,7 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
   const int b0 = blockIdx.x;
   int par = 0;  // table copy of the current round
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    // has this thread met |a_pq| >= 1e-8 sqrt(|a_pp a_qq|) this sweep?  (identical in every
+    // has this thread met |a_pq| >= 2^-30 sqrt(|a_pp a_qq|) this sweep?  (identical in every
     // block, since every block computes every rotation)
     int unconv = 0;
     for (int r = 0; r < kk - 1; ++r) {
@@ -996,10 +1075,12 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
         rr_pair(kk, r, b, pb, qb);
         const double app = __ldcg(&rdiag[par * kk + pb]), aqq = __ldcg(&rdiag[par * kk + qb]),
                      apq = __ldcg(&roff[par * kk + pb]);
-        const double a2 = apq * apq, sc2 = fabs(app * aqq);
-        unconv |= (apq != 0.0 && a2 >= 1e-16 * sc2);
+        // a_pq^2 against a_pp a_qq by exponents alone (within a factor of 4, no FP64 operation)
+        const int gap = exp_bits(app) + exp_bits(aqq) - 2 * exp_bits(apq);
+        const bool nz = (__double_as_longlong(apq) & 0x7FFFFFFFFFFFFFFFll) != 0;
+        unconv |= nz && gap <= 60;
         double c = 1.0, sn = 0.0;
-        if (apq != 0.0 && a2 > 1e-30 * sc2) jacobi_rotation(app, aqq, apq, c, sn);
+        if (nz && gap < 100) jacobi_rotation(app, aqq, apq, c, sn);
         cs[pb][0] = c; cs[pb][1] = sn;
         cs[qb][0] = c; cs[qb][1] = sn;
       }
@@ -1024,9 +1105,7 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
           double ajp, ajq;
           if (first) { ajp = c2 * rp[x] - s2 * rp[y]; ajq = c2 * rq[x] - s2 * rq[y]; }
           else { ajp = s2 * rp[y] + c2 * rp[x]; ajq = s2 * rq[y] + c2 * rq[x]; }
-          double np = c * ajp - sn * ajq, nq = sn * ajp + c * ajq;
-          if (x == q) np = 0.0;  // annihilated entry
-          if (x == p) nq = 0.0;
+          const double np = c * ajp - sn * ajq, nq = sn * ajp + c * ajq;
           A[(size_t)p * kk + x] = np;
           A[(size_t)q * kk + x] = nq;
           Vt[(size_t)p * kk + x] = c * vp[u] - sn * vq[u];
@@ -1085,40 +1164,74 @@ int jacobi_eig(int k, const double *H, int ldh, double *theta, double *S, int ld
 // and (max |V|, its row, its sign) for the sign convention.  Partials per row chunk.
 constexpr int kRRows = 512;
 
-__global__ void ritz_partial_kernel(int64_t n, int k, const double *V, const double *AV, const double *BV, int ld,
-                                    const double *theta, double *work) {
-  const int c = blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= k) return;
+// Block 32 columns x 8 row lanes (a thread per column over all 512 rows of a chunk was a chain of
+// loads: 68,921 rows, 160 columns 287 us, and 80 us for the sum over the chunks; now 156 and 23 us,
+// of which the FP64 operations 90 us).
+struct RitzSums {
+  double s0, s1, s2, amax, sgn, arow;
+  __device__ __forceinline__ void add(const RitzSums &o) {
+    s0 += o.s0; s1 += o.s1; s2 += o.s2;
+    if (o.amax > amax || (o.amax == amax && o.arow < arow)) { amax = o.amax; sgn = o.sgn; arow = o.arow; }
+  }
+};
+// Sum of the block's 8 row lanes per column, valid in lane 0.
+__device__ __forceinline__ RitzSums ritz_block_sum(const RitzSums &m) {
+  __shared__ RitzSums sm[8][33];
+  sm[threadIdx.y][threadIdx.x] = m;
+  __syncthreads();
+  RitzSums r = sm[0][threadIdx.x];
+  for (int y = 1; y < 8; ++y) r.add(sm[y][threadIdx.x]);
+  return r;
+}
+__global__ void __launch_bounds__(256) ritz_partial_kernel(int64_t n, int k, const double *V, const double *AV,
+                                                           const double *BV, int ld, const double *theta,
+                                                           double *work) {
+  const int c = blockIdx.y * 32 + threadIdx.x;
   const int64_t r0 = (int64_t)blockIdx.x * kRRows;
   const int64_t r1 = (r0 + kRRows < n) ? r0 + kRRows : n;
-  const double th = theta[c];
-  double s0 = 0, s1 = 0, s2 = 0, amax = -1.0, sgn = 1.0, arow = 0;
-  for (int64_t i = r0; i < r1; ++i) {
-    const double av = AV[i * ld + c], bv = BV[i * ld + c], v = V[i * ld + c];
-    const double rr = fma(-th, bv, av);
-    s0 = fma(rr, rr, s0);
-    s1 = fma(av, av, s1);
-    s2 = fma(v, bv, s2);
-    if (fabs(v) > amax) { amax = fabs(v); sgn = v < 0 ? -1.0 : 1.0; arow = (double)i; }
+  RitzSums m{0.0, 0.0, 0.0, -1.0, 1.0, (double)n};
+  if (c < k) {
+    const double th = theta[c];
+    long long top = -1, at = -1;
+    bool neg = false;
+#pragma unroll 4
+    for (int64_t i = r0 + threadIdx.y; i < r1; i += 8) {
+      const double av = AV[i * ld + c], bv = BV[i * ld + c], v = V[i * ld + c];
+      const double rr = fma(-th, bv, av);
+      m.s0 = fma(rr, rr, m.s0);
+      m.s1 = fma(av, av, m.s1);
+      m.s2 = fma(v, bv, m.s2);
+      // |v| > amax on the bits (FP64 compares run on the FP64 pipe, which bounds this loop)
+      const long long vb = __double_as_longlong(v), ab = vb & 0x7FFFFFFFFFFFFFFFll;
+      if (ab > top && ab <= 0x7FF0000000000000ll) { top = ab; neg = vb < 0; at = i; }
+    }
+    if (at >= 0) {
+      m.amax = __longlong_as_double(top);
+      m.sgn = neg && top != 0 ? -1.0 : 1.0;
+      m.arow = (double)at;
+    }
   }
+  const RitzSums r = ritz_block_sum(m);
+  if (threadIdx.y != 0 || c >= k) return;
   double *o = work + ((size_t)blockIdx.x * k + c) * 6;
-  o[0] = s0; o[1] = s1; o[2] = s2; o[3] = amax; o[4] = sgn; o[5] = arow;
+  o[0] = r.s0; o[1] = r.s1; o[2] = r.s2; o[3] = r.amax; o[4] = r.sgn; o[5] = r.arow;
 }
 
-__global__ void ritz_final_kernel(int k, int nchunks, const double *theta, const double *work, double *res,
-                                  double *res_paper, double *sgn) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= k) return;
-  double s0 = 0, s1 = 0, s2 = 0, amax = -1.0, sg = 1.0;
-  for (int z = 0; z < nchunks; ++z) {
-    const double *o = work + ((size_t)z * k + c) * 6;
-    s0 += o[0]; s1 += o[1]; s2 += o[2];
-    if (o[3] > amax) { amax = o[3]; sg = o[4]; }  // strict: the first row wins ties
-  }
-  const double rn = sqrt(s0);
-  res[c] = s1 > 0 ? rn / sqrt(s1) : INFINITY;
-  if (res_paper) res_paper[c] = (s2 > 0 && theta[c] != 0) ? rn / (fabs(theta[c]) * sqrt(s2)) : INFINITY;
-  if (sgn) sgn[c] = sg;
+__global__ void __launch_bounds__(256) ritz_final_kernel(int k, int nchunks, const double *theta, const double *work,
+                                                         double *res, double *res_paper, double *sgn) {
+  const int c = blockIdx.x * 32 + threadIdx.x;
+  RitzSums m{0.0, 0.0, 0.0, -1.0, 1.0, INFINITY};
+  if (c < k)
+    for (int z = threadIdx.y; z < nchunks; z += 8) {
+      const double *o = work + ((size_t)z * k + c) * 6;
+      m.add(RitzSums{o[0], o[1], o[2], o[3], o[4], o[5]});  // the first row wins ties
+    }
+  const RitzSums r = ritz_block_sum(m);
+  if (threadIdx.y != 0 || c >= k) return;
+  const double rn = sqrt(r.s0);
+  res[c] = r.s1 > 0 ? rn / sqrt(r.s1) : INFINITY;
+  if (res_paper) res_paper[c] = (r.s2 > 0 && theta[c] != 0) ? rn / (fabs(theta[c]) * sqrt(r.s2)) : INFINITY;
+  if (sgn) sgn[c] = r.sgn;
 }
 
 size_t ritz_work_doubles(int64_t n, int k) { return (size_t)((n + kRRows - 1) / kRRows) * k * 6; }
@@ -1127,9 +1240,9 @@ void ritz_residuals(int64_t n, int k, const double *V, const double *AV, const d
                     const double *theta, double *res, double *res_paper, double *sgn, double *work, cudaStream_t st) {
   if (k <= 0) return;
   const int nchunks = (int)((n + kRRows - 1) / kRRows);
-  dim3 grid(nchunks, (k + 127) / 128);
-  ritz_partial_kernel<<<grid, 128, 0, st>>>(n, k, V, AV, BV, ld, theta, work);
-  ritz_final_kernel<<<(k + 127) / 128, 128, 0, st>>>(k, nchunks, theta, work, res, res_paper, sgn);
+  dim3 grid(nchunks, (k + 31) / 32);
+  ritz_partial_kernel<<<grid, dim3(32, 8), 0, st>>>(n, k, V, AV, BV, ld, theta, work);
+  ritz_final_kernel<<<(k + 31) / 32, dim3(32, 8), 0, st>>>(k, nchunks, theta, work, res, res_paper, sgn);
 }
 
 // ------------------------------------------------------------------------------ locking

@@ -12,7 +12,7 @@ void spmm_real(int64_t n, const int64_t *rowptr, const int32_t *col, const doubl
                cudaStream_t st, const int *run_if = nullptr);
 // YB = B X in FP32 arithmetic (FP64 storage): input of an FP32 Gram matrix.
 void spmm_b32(int64_t n, const int64_t *rowptr, const int32_t *col, const double *valB, const double *X, int ldx,
-              int k, double *YB, int ldy, cudaStream_t st);
+              int k, float *x32, double *YB, int ldy, cudaStream_t st);
 
 // YA = A X and YB = B X in FP32 arithmetic (FP64 storage): the start of the FP32 solves.
 void spmm_ab32(int64_t n, const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB,
@@ -41,7 +41,7 @@ size_t gram_work_doubles(int64_t n, int k1, int k2);
 // fp32: FP32 inputs and accumulation within row chunks (for passes whose error a later
 // FP64 pass removes); run_if: device flag, the launch does nothing while *run_if == 0.
 void gram(int64_t n, const double *X, int ldx, int k1, const double *Y, int ldy, int k2, double *C, int ldc,
-          bool sym, double *work, cudaStream_t st, bool fp32 = false, const int *run_if = nullptr);
+          bool sym, double *work, cudaStream_t st, float *f32 = nullptr, const int *run_if = nullptr);
 
 // Z = alpha X S + beta Z;  X n x k1, S k1 x k2 (row-major, lds), Z n x k2.  upper: S is
 // upper triangular.  Z must not alias X.

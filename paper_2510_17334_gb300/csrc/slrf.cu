@@ -266,7 +266,6 @@ static void drop_bricks(slrf_ctx *ctx) {
   ctx->bricks = Bricks{};
 }
 static void drop_groups(slrf_ctx *ctx) {
-  drop_bricks(ctx);
   dfree(ctx, ctx->gptr);
   dfree(ctx, ctx->grec);
   dfree(ctx, ctx->grec64);
@@ -427,7 +426,7 @@ static void mesh_strides(const std::vector<int32_t> &cols, int64_t row, int64_t 
 // kernel stays.
 static int build_bricks(slrf_ctx *ctx) {
   drop_bricks(ctx);
-  if (!ctx->mixed || ctx->grp != 2) return SLRF_OK;
+  if (!ctx->mixed) return SLRF_OK;
   const int64_t n = ctx->n;
   std::vector<int64_t> rp((size_t)n + 1);
   if (cudaMemcpyAsync(rp.data(), ctx->rowptr, rp.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->st) !=
@@ -520,6 +519,15 @@ static int build_bricks(slrf_ctx *ctx) {
   dfree(ctx, stats);
   if (!fit) return give_up(SLRF_OK);
   ctx->bricks = B;
+  return SLRF_OK;
+}
+
+// Bricks for the COCG SpMM if the pattern has them, with pairs of rows (records) for the real
+// products; otherwise the groups stay as they are.
+static int use_bricks(slrf_ctx *ctx) {
+  int rc = build_bricks(ctx);
+  if (rc != SLRF_OK || ctx->bricks.count == 0) return rc;
+  if (ctx->grp != 2 && (rc = build_groups(ctx, 2)) != SLRF_OK) return rc;
   ctx->vec = cocg_vec_csr<float>();  // 64-entry tiles
   return SLRF_OK;
 }
@@ -532,7 +540,8 @@ static int setup_groups(slrf_ctx *ctx) {
   }
   int rc = build_groups(ctx, G);
   if (rc != SLRF_OK) return rc;
-  if (ctx->o.group == 0 && (rc = build_bricks(ctx)) != SLRF_OK) return rc;
+  // bricks before groups of any height, but for vector-valued pencils (B-diagonal records)
+  if (ctx->o.group == 0 && !ctx->bdiag && (rc = use_bricks(ctx)) != SLRF_OK) return rc;
   // the batched kernels run bricks or plain CSR, at the CSR lane width
   if (ctx->batched && ctx->bricks.count == 0) drop_groups(ctx);
   return SLRF_OK;
@@ -893,17 +902,20 @@ static int autotune_rows(slrf_ctx *ctx) {
     bool best_bricks = false;
     for (int g = 1; g <= 4; ++g) {
       if (g > 1 && !ctx->mixed && g != g_model) continue;
+      drop_bricks(ctx);
       if ((rc = build_groups(ctx, g)) != SLRF_OK) break;
       ctx->rpb_tuned = 0;
       if ((rc = time_spmm(t)) != SLRF_OK) break;
       if (t < best) { best = t; best_g = g; best_bricks = false; }
-      if ((rc = build_bricks(ctx)) != SLRF_OK) break;
+      if (g != 2) continue;
+      if ((rc = use_bricks(ctx)) != SLRF_OK) break;
       if (ctx->bricks.count == 0) continue;
       if ((rc = time_spmm(t)) != SLRF_OK) break;
       if (t < best) { best = t; best_g = g; best_bricks = true; }
     }
+    drop_bricks(ctx);
     if (rc == SLRF_OK) rc = build_groups(ctx, best_g);
-    if (rc == SLRF_OK && best_bricks) rc = build_bricks(ctx);
+    if (rc == SLRF_OK && best_bricks) rc = use_bricks(ctx);
     if (rc != SLRF_OK) {
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
@@ -965,8 +977,10 @@ static void tsgram(slrf_ctx *ctx, int64_t n, const double *X, int ldx, int k1, c
             run_if);
     ctx->launches += same ? 4 : 6;
   } else {
-    gram(n, X, ldx, k1, Y, ldy, k2, C, ldc, sym, ctx->work, ctx->st, fp32, run_if);
-    ctx->launches += 2;
+    // FP32: copies of both operands in a block that the outer update writes only at its end
+    gram(n, X, ldx, k1, Y, ldy, k2, C, ldc, sym, ctx->work, ctx->st, fp32 ? reinterpret_cast<float *>(ctx->BVt) : nullptr,
+         run_if);
+    ctx->launches += fp32 ? 4 : 2;
   }
 }
 static void tsgemm(slrf_ctx *ctx, int64_t n, const double *X, int ldx, int k1, const double *S, int lds, int k2,
@@ -1012,8 +1026,10 @@ static int rr_impl(slrf_ctx *ctx, double *U, int k, const double *X, const doubl
   if (ctx->mixed && ctx->grp > 1)
     spmm_grp_real32(n, ctx->grp, ctx->ngroups, ctx->gptr, ctx->grec, ctx->iflags + 15, grp_real_blocks(ctx), U, L,
                     k, ctx->dsqrt, ctx->x32, nullptr, ctx->BU, L, ctx->dsqrt, st, ctx->bdiag != 0);
-  else
-    spmm_b32(n, ctx->rowptr, ctx->col, ctx->valB, U, L, k, ctx->BU, L, st);
+  else {
+    ctx->launches += 1;  // the FP32 copy of U, in a block that is written only later
+    spmm_b32(n, ctx->rowptr, ctx->col, ctx->valB, U, L, k, reinterpret_cast<float *>(ctx->AVt), ctx->BU, L, st);
+  }
   cudaMemsetAsync(ctx->iflags + 11, 0, sizeof(int), st);
   tsgram(ctx, n, U, L, k, ctx->BU, L, k, ctx->Gm, k, true, true);
   chol_inv(k, ctx->Gm, k, ctx->Rinv, k, ctx->iflags + 11, st, nullptr, true);
