@@ -45,7 +45,7 @@
 #define SLRF_GRP_MINB 2
 #endif
 #ifndef SLRF_GRP_UNROLL_BD
-#define SLRF_GRP_UNROLL_BD 4
+#define SLRF_GRP_UNROLL_BD 9
 #endif
 // Per-record check of the gathered column in the grouped SpMM (1), or none (0): the records
 // are built on the device from a pattern validated at setup and checked once after the
@@ -772,8 +772,9 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
                                          const int *xo = nullptr) {
   static_assert(U == 0 || (BD && sizeof(R) == 8), "single columns: FP64 B-diagonal records");
   constexpr int VEC = U > 0 ? U : V;
-  constexpr int RS = grec_bytes<R, G, BD>();
+  constexpr int RS = BD ? 4 * (int)sizeof(R) : grec_bytes<R, G>();  // a record's values (general: and column)
   constexpr int CH = grp_chunk<R, BD>();
+  constexpr int CB = (int)grec_span<R, G, BD>(CH);  // bytes of a chunk
   static_assert(!BD || (G == 3 && CH % 3 == 0), "B-diagonal records: 3-row groups, whole triples per chunk");
   using C = cx_t<R>;
   const int lane = threadIdx.x & 31;
@@ -805,9 +806,10 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
       // the lanes' shared-memory reads of this buffer (ordered by the __syncwarp before
       // the call) precede the asynchronous proxy's writes
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      if (cnt > 0) {
-        mbar_expect_tx(bar + b, (uint32_t)(cnt * RS));
-        bulk_g2s(sbuf + (size_t)b * CH * RS, grec + (size_t)e0 * RS, (uint32_t)(cnt * RS), bar + b);
+      if (cnt > (BD ? 2 : 0)) {
+        const uint32_t bytes = (uint32_t)grec_span<R, G, BD>(cnt);
+        mbar_expect_tx(bar + b, bytes);
+        bulk_g2s(sbuf + (size_t)b * CB, grec + grec_span<R, G, BD>(e0), bytes, bar + b);
       } else {
         mbar_arrive(bar + b);
       }
@@ -836,17 +838,22 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
     if (b) ph1 ^= 1u; else ph0 ^= 1u;
     int cnt;
     first(cg, cc, cnt);
-    const unsigned char *rb_ = sbuf + (size_t)b * CH * RS;
+    const unsigned char *rb_ = sbuf + (size_t)b * CB;
     if constexpr (BD) {
-      // whole node triples: record t + d holds column 3J + d, whose B value belongs to row d
-      // (a malformed tail shorter than a triple is skipped, never read past the chunk)
+      // whole node triples: record d of a triple holds column 3J + d, whose B value belongs to row
+      // d (a malformed tail shorter than a triple is neither copied nor read).  The unrolled loop
+      // lets the compiler keep as many gathers in flight as the registers hold: 9 triples, a third
+      // of an interior node's, measured 4.97 ms against 5.08 at 4 and 5.47 at 3 (64 x 64 x 32 box,
+      // 128 columns)
 #pragma unroll kGrpUnrollBD
       for (int t = 0; t + 2 < cnt; t += 3) {
+        const unsigned char *const tp = rb_ + t / 3 * triple_bytes<R>();
+        const char *const x3 =
+            xlane + (unsigned long long)(unsigned)*reinterpret_cast<const int *>(tp + 3 * RS) * xbytes;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const unsigned char *rp = rb_ + (t + d) * RS;
-          const int c = *reinterpret_cast<const int *>(rp + grec_col<R, G, true>());
-          const char *const xc = xlane + (unsigned long long)(unsigned)c * xbytes;
+          const unsigned char *rp = tp + d * RS;
+          const char *const xc = x3 + (unsigned long long)d * xbytes;
           if constexpr (U > 0) {
             const double2 r01 = reinterpret_cast<const double2 *>(rp)[0];  // a0, a1
             const double2 r23 = reinterpret_cast<const double2 *>(rp)[1];  // a2, b
@@ -976,14 +983,22 @@ __device__ __forceinline__ void grp_walk(const int64_t ngroups, const int64_t *_
 template <typename R, int V, int G, bool BD, bool FRESH>
 __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const int rb, const int tile) {
   constexpr int VEC = V;
-  constexpr int RS = grec_bytes<R, G, BD>();
   using C = cx_t<R>;
   extern __shared__ __align__(128) unsigned char grp_smem[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w_tile0 = tile * 32 * VEC;
   const int w0 = w_tile0 + lane_w<V>(lane);
-  // (beta and the poles are read again in each group's epilogue: not held across the walk)
+  // beta and the poles of the tile in the working precision (read in each group's epilogue: not
+  // held across the walk, not converted from FP64 again for every group)
+  constexpr int TW = 32 * VEC;
+  __shared__ C s_be[TW], s_sg[TW];
+  for (int t = threadIdx.x; t < TW; t += kThreads) {
+    s_be[t] = to_c<R>(a.ws[w_tile0 + t].beta);
+    s_sg[t] = a.sig[(w_tile0 + t) & (a.mp - 1)];
+  }
+  __syncthreads();
+  const int lw = lane_w<V>(lane);
   bool any_act = false;
 #pragma unroll
   for (int v = 0; v < VEC; ++v) any_act |= a.ws[w0 + woff<V>(v)].active != 0;
@@ -1003,8 +1018,8 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
       C sg[VEC], be[VEC];
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {
-        be[v] = to_c<R>(a.ws[w0 + woff<V>(v)].beta);
-        sg[v] = a.sig[(w0 + woff<V>(v)) & (a.mp - 1)];
+        be[v] = s_be[lw + woff<V>(v)];
+        sg[v] = s_sg[lw + woff<V>(v)];
       }
 #pragma unroll
       for (int j = 0; j < G; ++j) {
@@ -1034,7 +1049,7 @@ __device__ __forceinline__ void cocg_spmm_grp_body(const CocgArgs<R> &a, const i
     };
     grp_walk<R, VEC, G, BD>(a.ngroups, a.gptr, a.grec, a.err, a.n, gfirst, gstride,
                             reinterpret_cast<const char *>(a.r + w0), (unsigned)a.W * (unsigned)sizeof(C),
-                            grp_smem + (size_t)warp * 2 * grp_chunk<R, BD>() * RS, s_bar[warp], epi);
+                            grp_smem + (size_t)warp * 2 * grec_span<R, G, BD>(grp_chunk<R, BD>()), s_bar[warp], epi);
   }
   spmm_tail<R, VEC>(a, acc, w_tile0, rb, tile, a.nrb);
 }
@@ -1328,8 +1343,13 @@ __global__ void grp_check_kernel(int64_t n, int64_t ngroups, const int64_t *__re
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ngroups; g += stride)
     if (gptr[g] < 0 || gptr[g + 1] < gptr[g] || (BD && (gptr[g + 1] - gptr[g]) % 3 != 0)) atomicExch(flag, 1);
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nrec; e += stride) {
-    const int c = *reinterpret_cast<const int *>(rec + (size_t)e * grec_bytes<R, G, BD>() + grec_col<R, G, BD>());
-    if (c < 0 || (int64_t)c >= n) atomicExch(flag, 1);
+    if constexpr (BD) {
+      const int c = *reinterpret_cast<const int *>(rec + (size_t)(e / 3) * triple_bytes<R>() + 12 * sizeof(R));
+      if (c < 0 || (int64_t)c + 2 >= n) atomicExch(flag, 1);
+    } else {
+      const int c = *reinterpret_cast<const int *>(rec + (size_t)e * grec_bytes<R, G>() + grec_col<R, G>());
+      if (c < 0 || (int64_t)c >= n) atomicExch(flag, 1);
+    }
   }
 }
 template <typename R>
@@ -1378,25 +1398,18 @@ __global__ void grp_bd_detect_kernel(int64_t n, int64_t ngroups, const int64_t *
 }
 template <typename R>
 __global__ void grp_bd_convert_kernel(int64_t nrec, const unsigned char *__restrict__ rec, unsigned char *bdrec) {
-  constexpr int RS = grec_bytes<R, 3>(), RB = grec_bytes<R, 3, true>();
+  constexpr int RS = grec_bytes<R, 3>();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nrec) return;
   const unsigned char *rp = rec + (size_t)e * RS;
-  unsigned char *bp = bdrec + (size_t)e * RB;
   const int c = *reinterpret_cast<const int *>(rp + grec_col<R, 3>());
-  const int d = c % 3;
-  for (int t = 0; t < RB / 4; ++t) reinterpret_cast<int *>(bp)[t] = 0;
-  if constexpr (sizeof(R) == 8) {
-    const double *v = reinterpret_cast<const double *>(rp);
-    double *o = reinterpret_cast<double *>(bp);
-    o[0] = v[0]; o[1] = v[1]; o[2] = v[2]; o[3] = v[3 + d];
-  } else {
-    const float *v = reinterpret_cast<const float *>(rp);
-    float *o = reinterpret_cast<float *>(bp);
-    const int s = SLRF_GRP_SPLAT ? 2 : 1;
-    o[0] = v[0]; o[1] = v[s]; o[2] = v[2 * s]; o[3] = v[s * (3 + d)];
-  }
-  *reinterpret_cast<int *>(bp + grec_col<R, 3, true>()) = c;
+  const int d = (int)(e % 3);  // = c % 3 (grp_bd_detect)
+  unsigned char *const tp = bdrec + (size_t)(e / 3) * triple_bytes<R>();
+  const int s = sizeof(R) == 4 && SLRF_GRP_SPLAT ? 2 : 1;
+  const R *v = reinterpret_cast<const R *>(rp);
+  R *o = reinterpret_cast<R *>(tp) + 4 * d;
+  o[0] = v[0]; o[1] = v[s]; o[2] = v[2 * s]; o[3] = v[s * (3 + d)];
+  if (d == 0) *reinterpret_cast<int4 *>(tp + 12 * sizeof(R)) = make_int4(c, 0, 0, 0);
 }
 template <typename R>
 void grp_bd_detect(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *rec, int *flag, int blocks,
@@ -1670,7 +1683,6 @@ struct GrpReal32 {
 template <int G, bool BD>
 __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<float, kReal32Vec, G>())) spmm_grp_real32_kernel(const GrpReal32 a) {
   constexpr int VEC = kReal32Vec;
-  constexpr int RS = grec_bytes<float, G, BD>();
   extern __shared__ __align__(128) unsigned char grp_smem[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1700,7 +1712,7 @@ __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<float, kReal32Vec, G>
   };
   grp_walk<float, VEC, G, BD>(a.ngroups, a.gptr, a.grec, a.err, a.n, gfirst, gstride,
                               reinterpret_cast<const char *>(a.x + c0), (unsigned)a.ldx * 4u,
-                              grp_smem + (size_t)warp * 2 * grp_chunk<float, BD>() * RS, s_bar[warp], epi);
+                              grp_smem + (size_t)warp * 2 * grec_span<float, G, BD>(grp_chunk<float, BD>()), s_bar[warp], epi);
 }
 void spmm_grp_real32(int64_t n, int G, int64_t ngroups, const int64_t *gptr, const unsigned char *grec, int *err,
                      int nrb, const double *X, int ldx, int k, const double *xscale, float *x32, double *YA,
@@ -1752,7 +1764,6 @@ __global__ void to_f64_scaled_kernel(int64_t n, int k, const double *__restrict_
 }
 template <int U>
 __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<double, 1, 3>())) spmm_grp_real64_kernel(const GrpReal64 a) {
-  constexpr int RS = grec_bytes<double, 3, true>();
   extern __shared__ __align__(128) unsigned char grp_smem[];
   __shared__ __align__(8) uint64_t s_bar[kWarps][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1781,7 +1792,7 @@ __global__ void __launch_bounds__(kThreads, (cocg_grp_minb<double, 1, 3>())) spm
   };
   grp_walk<double, 1, 3, true, U>(a.ngroups, a.gptr, a.grec, a.err, a.n, gfirst, gstride,
                                   reinterpret_cast<const char *>(a.x), (unsigned)a.ldx * 8u,
-                                  grp_smem + (size_t)warp * 2 * grp_chunk<double, true>() * RS, s_bar[warp], epi, xo);
+                                  grp_smem + (size_t)warp * 2 * grec_span<double, 3, true>(grp_chunk<double, true>()), s_bar[warp], epi, xo);
 }
 void spmm_grp_real64(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *grec, int *err, int nrb,
                      const double *X, int ldx, int k, const double *xscale, double *x64, double *YA, double *YB,

@@ -91,7 +91,7 @@ struct CocgArgs {
   int64_t ngroups;
   const int64_t *gptr;       // [ngroups + 1]
   const unsigned char *grec; // records, 16-byte aligned
-  int bdiag;                 // 1: B-diagonal records (G = 3, see grec_col)
+  int bdiag;                 // 1: B-diagonal records (G = 3, see triple_bytes)
   Bricks bricks;             // FP32: staged SpMM instead of the two above (count > 0)
   int *err;                  // 1: a bounded wait gave up (SLRF_ETIMEOUT); 2, 3: group records
                              // inconsistent; 4: update buffers missing (SLRF_EINVAL)
@@ -114,19 +114,27 @@ struct CocgArgs {
 // B-diagonal records (BD, 3-row groups only): vector-valued FEM pencils whose B couples a dof
 // only with the same dof of a neighbour node (a mass matrix M (x) I_3) have, in a node's group,
 // one nonzero B value per column c -- the row c mod 3.  When every group's columns come in
-// aligned node triples (3J, 3J + 1, 3J + 2), a record holds the 3 A values, that one B value
-// and the column (FP32 32 B, FP64 48 B), and the walk knows the B row from the record's place
-// in its triple: one B product per record instead of three.  Checked on the device when the
-// records are built (grp_bd_detect); otherwise the general records are kept.
-template <typename R, int G, bool BD = false> __host__ __device__ constexpr int grec_col() {
-  return BD ? 4 * (int)sizeof(R) : ((sizeof(R) == 8 || SLRF_GRP_SPLAT) ? 16 * G : 8 * G);
+// aligned node triples (3J, 3J + 1, 3J + 2), the records are kept per triple: three times the 3
+// A values and that one B value, then the column 3J (FP32 64 B, FP64 112 B a triple; with a
+// column of its own in every record, 96 and 144 B, the 64 x 64 x 32 box read half as much more
+// records and the walk two more shared-memory words per triple), and the walk knows the B row
+// from the record's place in its triple: one B product per record instead of three.  Checked on
+// the device when the records are built (grp_bd_detect); otherwise the general records are kept.
+template <typename R, int G> __host__ __device__ constexpr int grec_col() {
+  return (sizeof(R) == 8 || SLRF_GRP_SPLAT) ? 16 * G : 8 * G;
 }
-template <typename R, int G, bool BD = false> __host__ __device__ constexpr int grec_bytes() {
-  return (grec_col<R, G, BD>() + 4 + 15) / 16 * 16;
+template <typename R, int G> __host__ __device__ constexpr int grec_bytes() {
+  return (grec_col<R, G>() + 4 + 15) / 16 * 16;
 }
-inline int grec_bytes_rt(int G, bool fp32, bool bd = false) {
-  const int col = bd ? (fp32 ? 16 : 32) : ((!fp32 || SLRF_GRP_SPLAT) ? 16 * G : 8 * G);
-  return (col + 4 + 15) / 16 * 16;
+template <typename R> __host__ __device__ constexpr int triple_bytes() { return 12 * (int)sizeof(R) + 16; }
+// Bytes of n records (whole triples of B-diagonal ones).
+template <typename R, int G, bool BD = false> __host__ __device__ constexpr int64_t grec_span(int64_t n) {
+  return BD ? n / 3 * triple_bytes<R>() : n * grec_bytes<R, G>();
+}
+inline int64_t grec_span_rt(int64_t n, int G, bool fp32, bool bd = false) {
+  if (bd) return n / 3 * (fp32 ? triple_bytes<float>() : triple_bytes<double>());
+  const int col = (!fp32 || SLRF_GRP_SPLAT) ? 16 * G : 8 * G;
+  return n * ((col + 4 + 15) / 16 * 16);
 }
 // Records per staged chunk (one bulk copy): 64 (2 KB of 32-byte FP32 records, 4 KB in FP64).
 #ifndef SLRF_GRP_CHUNK32
@@ -144,7 +152,7 @@ template <typename R, bool BD = false> __host__ __device__ constexpr int grp_chu
 }
 // Dynamic shared memory of the grouped SpMM: two chunk buffers per warp.
 template <typename R, int G, bool BD = false> __host__ __device__ constexpr int grp_smem_bytes() {
-  return kWarps * 2 * grp_chunk<R, BD>() * grec_bytes<R, G, BD>();
+  return kWarps * 2 * (int)grec_span<R, G, BD>(grp_chunk<R, BD>());
 }
 
 // Dynamic shared memory of the brick SpMM (at least its reduction's scratch).
@@ -239,7 +247,7 @@ void cocg_kernel_attrs();
 template <typename R>
 void grp_check(int64_t n, int G, int64_t ngroups, const int64_t *gptr, const unsigned char *rec, int *flag,
                int blocks, cudaStream_t st, bool bd = false);
-// B-diagonal records (see grec_col): *flag = 1 unless every group of 3 rows has its records
+// B-diagonal records (see triple_bytes): *flag = 1 unless every group of 3 rows has its records
 // in aligned column triples and B vanishes off the row c mod 3 (general records as input).
 template <typename R>
 void grp_bd_detect(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *rec, int *flag, int blocks,

@@ -93,7 +93,7 @@ struct slrf_ctx {
   int64_t launches = 0;              // kernels enqueued by the orchestration (statistics)
   int64_t rpb_tuned = 0;             // autotuned COCG rows per block (0 = default)
   int grp_bpsm = 0;                  // resident blocks per SM of the grouped SpMM in use
-  int bdiag = 0;                     // the grouped records are B-diagonal (see grec_col)
+  int bdiag = 0;                     // the grouped records are B-diagonal (see triple_bytes)
   Bricks bricks{};                   // mixed path: staged SpMM format (count 0: not in use)
   bool batched = false;              // a problem of a batch: lane width 2 in FP32
   unsigned char *grec64 = nullptr;   // mixed path: FP64 B-diagonal records of the same groups
@@ -257,7 +257,6 @@ static int group_counts(slrf_ctx *ctx, int G, std::vector<int> &cnt) {
   cudaFree(d);
   return e == cudaSuccess ? SLRF_OK : SLRF_ECUDA;
 }
-static int grec_size(int G, bool fp32) { return grec_bytes_rt(G, fp32); }
 static void drop_bricks(slrf_ctx *ctx) {
   dfree(ctx, const_cast<int4 *>(ctx->bricks.groups));
   dfree(ctx, const_cast<int *>(ctx->bricks.nrows));
@@ -289,7 +288,7 @@ static int build_groups(slrf_ctx *ctx, int G) {
   for (int64_t g = 0; g < ng; ++g) off[g + 1] = off[g] + cnt[g];
   // gptr[ng + 1] (one spare word) holds the record check's flag
   if ((rc = dalloc(ctx, &ctx->gptr, (size_t)ng + 2)) != SLRF_OK) return rc;
-  if ((rc = dalloc(ctx, &ctx->grec, (size_t)off[ng] * grec_size(G, ctx->mixed) + 16)) != SLRF_OK) return rc;
+  if ((rc = dalloc(ctx, &ctx->grec, (size_t)grec_span_rt(off[ng], G, ctx->mixed) + 16)) != SLRF_OK) return rc;
   if (cudaMemcpyAsync(ctx->gptr, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, ctx->st) !=
       cudaSuccess)
     return SLRF_ECUDA;
@@ -326,7 +325,7 @@ static int build_groups(slrf_ctx *ctx, int G) {
       return SLRF_ECUDA;
     if (nbd == 0) {
       unsigned char *bdrec = nullptr;
-      if ((rc = dalloc(ctx, &bdrec, (size_t)off[ng] * grec_bytes_rt(3, ctx->mixed, true) + 16)) != SLRF_OK) return rc;
+      if ((rc = dalloc(ctx, &bdrec, (size_t)grec_span_rt(off[ng], 3, ctx->mixed, true) + 16)) != SLRF_OK) return rc;
       if (ctx->mixed) grp_bd_convert<float>(off[ng], ctx->grec, bdrec, ctx->st);
       else grp_bd_convert<double>(off[ng], ctx->grec, bdrec, ctx->st);
       if (cudaMemsetAsync(dflag, 0, sizeof(int), ctx->st) != cudaSuccess) return SLRF_ECUDA;
@@ -346,8 +345,8 @@ static int build_groups(slrf_ctx *ctx, int G) {
       if (ctx->mixed) {
         // FP64 B-diagonal records of the same groups for the FP64 real products of the outer step
         unsigned char *gen64 = nullptr, *bd64 = nullptr;
-        if ((rc = dalloc(ctx, &gen64, (size_t)off[ng] * grec_bytes_rt(3, false) + 16)) != SLRF_OK) return rc;
-        if ((rc = dalloc(ctx, &bd64, (size_t)off[ng] * grec_bytes_rt(3, false, true) + 16)) != SLRF_OK) return rc;
+        if ((rc = dalloc(ctx, &gen64, (size_t)grec_span_rt(off[ng], 3, false) + 16)) != SLRF_OK) return rc;
+        if ((rc = dalloc(ctx, &bd64, (size_t)grec_span_rt(off[ng], 3, false, true) + 16)) != SLRF_OK) return rc;
         grp_fill<double>(ctx->n, 3, ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), ctx->gptr, gen64, ctx->st);
         grp_bd_convert<double>(off[ng], gen64, bd64, ctx->st);
         if (cudaMemsetAsync(dflag, 0, sizeof(int), ctx->st) != cudaSuccess) return SLRF_ECUDA;
