@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <utility>
 
 #include "../../include/slrf.h"
 #include "common.cuh"
@@ -218,21 +219,22 @@ int eig_grad_values(int64_t n, const int64_t *rowptr, const int32_t *col, int k,
 namespace slrf {
 
 struct MinresScal {
-  double beta, oldb, dbar, epsln, phibar, cs, sn, alfa, beta1;
-  double oldeps, delta, gamma, phi;
+  double beta, ib, oldb, dbar, epsln, phibar, cs, sn, beta1;  // ib = 1 / beta
+  double iob, oldeps, delta, ig, phi;  // of the pending w and x update: 1 / oldb, ..., 1 / gamma
   int active;   // 1 while the column still iterates
   int pending;  // 1: the w and x update of the last step is still to come
 };
 
-// One MINRES step is two launches: minres_apply_kernel (products with the Lanczos vector, the
-// recurrence's first half, alfa) and minres_update_kernel (its second half, beta, the Givens
-// step and the stopping test).  Blocks of a 32-column tile write partial column sums; the last
-// one adds them in a fixed order and updates the tile's scalars.  The Lanczos vectors rotate
-// through three buffers (no copies), v = r2 / beta is never stored (A v = (A r2) / beta), and
-// the w and x update of a step, which needs only the row's own entries, rides on the next
-// step's apply.  With 11 launches a step and column sums over chunks of 512 rows on one
-// thread each (230 us of latency for 2 x 4 blocks) a step of n = 2,002, k = 16 took 240 us;
-// now 26 us, two launch latencies with their last-block sums (384 steps: 96 -> 9.9 ms).
+// All steps between two looks at the convergence run in one cooperative launch
+// (minres_loop_kernel); a step is an apply phase (product with the Lanczos vector, first half of
+// the recurrence, alfa) and an update phase (second half, beta, Givens step, stopping test), with
+// a grid barrier per 32-column tile after each.  The blocks write partial column sums and every
+// block adds them itself in the same order, so nothing else is exchanged.  The Lanczos vectors
+// rotate through three buffers (no copies), v = r2 / beta is never stored (A v = (A r2) / beta),
+// and the w and x update of a step, which needs only the row's own entries, rides on the next
+// step's apply.  n = 2,002, k = 16: 11 launches a step and column sums of 512 rows on a thread
+// 240 us, two launches a step 26 us, now 16 us (two barriers, the latency of the gathers and
+// of the FP64 roots).
 constexpr int kAdjWarps = 8;
 
 // Sum v over the warps of the block and then over the blocks of the tile (gridDim.x of them):
@@ -291,6 +293,7 @@ __global__ void minres_init_kernel(int k, const double *b2, MinresScal *s) {
   MinresScal m{};
   m.beta1 = sqrt(b2[c]);
   m.beta = m.beta1;
+  m.ib = m.beta1 > 0.0 ? 1.0 / m.beta1 : 0.0;
   m.phibar = m.beta1;
   m.cs = -1.0;
   m.active = m.beta1 > 0.0 ? 1 : 0;
@@ -303,145 +306,191 @@ struct MinresArgs {
   const int64_t *rowptr;
   const int32_t *col;
   const double *valA, *valB, *lam;
-  const double *r1, *r2;  // Lanczos vectors of the last two steps (unscaled; beta = ||r2||)
-  double *y;              // the next one
-  const double *w;
-  double *w2, *x;
+  double *r1, *r2;  // Lanczos vectors of the last two steps (unscaled; beta = ||r2||)
+  double *y;        // the next one
+  double *w, *w2, *x;
   MinresScal *s;
-  double *part;
-  unsigned *counters;
+  double *part;        // two sets of [blocks][k] partial sums
+  unsigned *counters;  // one per tile
+  int *err;
   double tol;
+  int steps, cw;  // steps of this launch (0: only the pending updates); lanes per column group
 };
 
-// w and x of the previous step for one entry: w_new = (v - oldeps w2 - delta w) / gamma into w2
-// (the caller swaps the two), x += phi w_new, with v = r1 / oldb that step's Lanczos vector.
-struct MinresW {
-  double iob, oldeps, delta, ig, phi;
-  __device__ explicit MinresW(const MinresScal &m)
-      : iob(1.0 / m.oldb), oldeps(m.oldeps), delta(m.delta), ig(1.0 / m.gamma), phi(m.phi) {}
-  __device__ __forceinline__ void apply(const MinresArgs &a, int64_t t, double r1) const {
-    const double wn = fma(-delta, a.w[t], fma(-oldeps, a.w2[t], r1 * iob)) * ig;
-    a.w2[t] = wn;
-    a.x[t] = fma(phi, wn, a.x[t]);
-  }
-};
-
-// A warp takes a row at a time, cw lanes (8, 16 or 32) over the columns of the tile; with
-// fewer than 32 columns the 32 / cw lane groups share the row's entries.
-template <bool PRODUCT>
-__global__ void __launch_bounds__(32 * kAdjWarps) minres_apply_kernel(const MinresArgs a, int cw) {
-  __shared__ double2 s_ab[kAdjWarps][32];
-  __shared__ int s_c[kAdjWarps][32];
+// Sum over the blocks of the tile of their partial sums, the same in every block; scratch
+// [kAdjWarps][32].  Result in every warp's lane c.
+__device__ __forceinline__ double tile_sum(const double *part, int k, double (*sm)[32]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = lane & (cw - 1), part = lane / cw, parts = 32 / cw;
-  const int c = blockIdx.y * 32 + sub;
-  const bool ok = c < a.k;
-  MinresScal m{};
-  if (ok) m = a.s[c];
-  const bool act = PRODUCT && ok && m.active != 0, pend = ok && m.pending != 0;
-  // nothing left to do in this tile (the same for every block: the scalars change only after
-  // all blocks of a launch have arrived)
-  if (!__syncthreads_or(act || pend)) return;
-  const bool own = part == 0;
-  const MinresW wx(m);
-  const double ib = 1.0 / m.beta, ratio = m.oldb > 0.0 ? m.beta / m.oldb : 0.0;
-  const double lam = act ? a.lam[c] : 0.0;
-  const bool any = __any_sync(0xffffffffu, act);
-  const char *const xl = reinterpret_cast<const char *>(a.r2 + (ok ? c : 0));
-  const unsigned row_bytes = (unsigned)a.k * (unsigned)sizeof(double);
-  double sum = 0.0;
-  const int64_t i0 = (int64_t)blockIdx.x * a.rows, i1 = i0 + a.rows < a.n ? i0 + a.rows : a.n;
-  for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) {
-    const int64_t t = i * a.k + c;
-    double sa = 0.0, sb = 0.0, r1 = 0.0, r2 = 0.0;
-    if (own && ok) {
-      if (pend || (act && m.oldb > 0.0)) r1 = a.r1[t];
-      if (act) r2 = a.r2[t];
-    }
-    if (any) {
-      const int64_t rs = a.rowptr[i], re = a.rowptr[i + 1];
-      for (int64_t e0 = rs; e0 < re; e0 += 32) {
-        const int cnt = (int)(re - e0 < 32 ? re - e0 : 32);
-        __syncwarp();
-        if (lane < cnt) {
-          s_c[warp][lane] = a.col[e0 + lane];
-          s_ab[warp][lane] = make_double2(a.valA[e0 + lane], a.valB[e0 + lane]);
-        }
-        __syncwarp();
-#pragma unroll 4
-        for (int q = part; q < cnt; q += parts) {
-          const double2 ab = s_ab[warp][q];
-          const double x =
-              *reinterpret_cast<const double *>(xl + (unsigned long long)(unsigned)s_c[warp][q] * row_bytes);
-          sa = fma(ab.x, x, sa);
-          sb = fma(ab.y, x, sb);
-        }
-      }
-      for (int o = cw; o < 32; o <<= 1) {
-        sa += __shfl_xor_sync(0xffffffffu, sa, o);
-        sb += __shfl_xor_sync(0xffffffffu, sb, o);
-      }
-    }
-    if (own && ok) {
-      if (pend) wx.apply(a, t, r1);
-      if (act) {
-        const double y = fma(-lam, sb, sa) * ib - ratio * r1;
-        a.y[t] = y;
-        sum = fma(r2 * ib, y, sum);
-      }
-    }
+  const int c = blockIdx.y * 32 + lane;
+  double s = 0.0;
+  if (c < k) {
+#pragma unroll 8
+    for (unsigned b = warp; b < gridDim.x; b += kAdjWarps) s += __ldcg(part + (size_t)b * k + c);
   }
-  double alfa;
-  if (!tile_reduce(sum, a.k, a.part, a.counters, alfa)) return;
-  if (warp == 0 && own && ok) {
-    MinresScal &g = a.s[c];
-    g.alfa = alfa;
-    g.pending = 0;
+  __syncthreads();
+  sm[warp][lane] = s;
+  __syncthreads();
+  s = 0.0;
+#pragma unroll
+  for (int w = 0; w < kAdjWarps; ++w) s += sm[w][lane];
+  return s;
+}
+// This block's partial sum of v over its warps.
+__device__ __forceinline__ void block_part(double v, double *part, int k, double (*sm)[32]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.y * 32 + lane;
+  __syncthreads();
+  sm[warp][lane] = v;
+  __syncthreads();
+  if (warp == 0 && c < k) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kAdjWarps; ++w) s += sm[w][lane];
+    part[(size_t)blockIdx.x * k + c] = s;
   }
 }
 
-// y -= (alfa / beta) r2; beta_new = ||y||; Givens step; the column stops once
-// phibar <= tol beta1 (its state is frozen after the pending w and x update).
-__global__ void __launch_bounds__(32 * kAdjWarps) minres_update_kernel(const MinresArgs a) {
+// A warp takes a row at a time, cw lanes (8, 16 or 32) over the columns of the tile; with
+// fewer than 32 columns the 32 / cw lane groups share the row's entries.  A row's own entries
+// are always read and written by the same thread; only the gathered rows of r2 come from other
+// blocks, after the barrier's acquire.
+__global__ void __launch_bounds__(32 * kAdjWarps) minres_loop_kernel(const MinresArgs a) {
+  __shared__ double2 s_ab[kAdjWarps][32];
+  __shared__ int s_c[kAdjWarps][32];
+  __shared__ double sm[kAdjWarps][32];
+  __shared__ MinresScal sc[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c = blockIdx.y * 32 + lane;
-  const bool ok = c < a.k;
-  MinresScal m{};
-  if (ok) m = a.s[c];
-  const bool act = ok && m.active != 0;
-  if (!__syncthreads_or(act)) return;
-  const double ratio = act && m.beta > 0.0 ? m.alfa / m.beta : 0.0;
-  double sum = 0.0;
+  const int sub = lane & (a.cw - 1), group = lane / a.cw, groups = 32 / a.cw;
+  const int c = blockIdx.y * 32 + sub;
+  const bool ok = c < a.k, own = group == 0;
+  const int cl = blockIdx.y * 32 + lane;  // this lane's column where all lanes take columns
+  if (warp == 0) sc[lane] = cl < a.k ? a.s[cl] : MinresScal{};
+  __syncthreads();
+  double *r1 = a.r1, *r2 = a.r2, *y = a.y, *w = a.w, *w2 = a.w2;
+  double *const partA = a.part, *const partB = a.part + (size_t)gridDim.x * a.k;
+  const double lam = ok ? a.lam[c] : 0.0;
+  const unsigned row_bytes = (unsigned)a.k * (unsigned)sizeof(double);
   const int64_t i0 = (int64_t)blockIdx.x * a.rows, i1 = i0 + a.rows < a.n ? i0 + a.rows : a.n;
-  if (act) {
-#pragma unroll 4
+  GridBarrier gb{a.counters + blockIdx.y, a.err};
+  unsigned epoch = 0;
+  for (int step = 0;; ++step) {
+    const bool last = step == a.steps;  // past the steps of this launch: nothing more, but with
+                                        // steps = 0 the pending updates
+    if (last && a.steps > 0) break;
+    const MinresScal m = sc[sub];
+    const bool act = ok && !last && m.active != 0, pend = ok && m.pending != 0;
+    // the same in every block of the tile
+    const bool more = __syncthreads_or(act) != 0;
+    if (!more && !__syncthreads_or(pend)) break;
+    // apply: y = (A r2 - lambda B r2) / beta - (beta / oldb) r1, alfa = v^T y
+    const double ratio = m.oldb > 0.0 ? m.beta * m.iob : 0.0;
+    const bool any = __any_sync(0xffffffffu, act);
+    const char *const xl = reinterpret_cast<const char *>(r2 + (ok ? c : 0));
+    double sum = 0.0;
     for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) {
       const int64_t t = i * a.k + c;
-      const double y = a.y[t] - ratio * a.r2[t];
-      a.y[t] = y;
-      sum = fma(y, y, sum);
+      double sa = 0.0, sb = 0.0, o1 = 0.0, o2 = 0.0;
+      if (own && ok) {
+        if (pend || (act && m.oldb > 0.0)) o1 = r1[t];
+        if (act) o2 = r2[t];
+      }
+      if (any) {
+        const int64_t rs = a.rowptr[i], re = a.rowptr[i + 1];
+        for (int64_t e0 = rs; e0 < re; e0 += 32) {
+          const int cnt = (int)(re - e0 < 32 ? re - e0 : 32);
+          __syncwarp();
+          if (lane < cnt) {
+            s_c[warp][lane] = a.col[e0 + lane];
+            s_ab[warp][lane] = make_double2(a.valA[e0 + lane], a.valB[e0 + lane]);
+          }
+          __syncwarp();
+#pragma unroll 4
+          for (int q = group; q < cnt; q += groups) {
+            const double2 ab = s_ab[warp][q];
+            const double x =
+                *reinterpret_cast<const double *>(xl + (unsigned long long)(unsigned)s_c[warp][q] * row_bytes);
+            sa = fma(ab.x, x, sa);
+            sb = fma(ab.y, x, sb);
+          }
+        }
+        for (int o = a.cw; o < 32; o <<= 1) {
+          sa += __shfl_xor_sync(0xffffffffu, sa, o);
+          sb += __shfl_xor_sync(0xffffffffu, sb, o);
+        }
+      }
+      if (own && ok) {
+        if (pend) {  // w_new = (v - oldeps w2 - delta w) / gamma, x += phi w_new (v = r1 / oldb)
+          const double wn = fma(-m.delta, w[t], fma(-m.oldeps, w2[t], o1 * m.iob)) * m.ig;
+          w2[t] = wn;
+          a.x[t] = fma(m.phi, wn, a.x[t]);
+        }
+        if (act) {
+          const double yy = fma(-lam, sb, sa) * m.ib - ratio * o1;
+          y[t] = yy;
+          sum = fma(o2 * m.ib, yy, sum);
+        }
+      }
     }
+    if (!more) {
+      __syncthreads();
+      if (warp == 0) sc[lane].pending = 0;
+      __syncthreads();
+      break;
+    }
+    block_part(own && ok ? sum : 0.0, partA, a.k, sm);
+    if (!grid_sync(gb, gridDim.x, epoch)) return;
+    const double alfa = tile_sum(partA, a.k, sm);  // lane c: column c
+    // update: y -= (alfa / beta) r2, beta = ||y||
+    const MinresScal ml = sc[lane];
+    const bool actl = cl < a.k && ml.active != 0;
+    const double f = actl ? alfa * ml.ib : 0.0;
+    sum = 0.0;
+    if (actl) {
+#pragma unroll 4
+      for (int64_t i = i0 + warp; i < i1; i += kAdjWarps) {
+        const int64_t t = i * a.k + cl;
+        const double yy = y[t] - f * r2[t];
+        y[t] = yy;
+        sum = fma(yy, yy, sum);
+      }
+    }
+    block_part(sum, partB, a.k, sm);
+    if (!grid_sync(gb, gridDim.x, epoch)) return;
+    const double b2 = tile_sum(partB, a.k, sm);
+    if (warp == 0) {
+      MinresScal g = ml;
+      g.pending = 0;
+      if (actl) {
+        g.oldb = g.beta;
+        g.iob = g.ib;
+        g.ib = b2 > 0.0 ? rsqrt(b2) : 0.0;
+        g.beta = b2 * g.ib;
+        g.oldeps = g.epsln;
+        g.delta = g.cs * g.dbar + g.sn * alfa;
+        const double gbar = g.sn * g.dbar - g.cs * alfa;
+        g.epsln = g.sn * g.beta;
+        g.dbar = -g.cs * g.beta;
+        const double g2 = fma(gbar, gbar, b2);  // gamma^2
+        g.ig = g2 > 0.0 ? rsqrt(g2) : 1e300;
+        g.cs = gbar * g.ig;
+        g.sn = g.beta * g.ig;
+        g.phi = g.cs * g.phibar;
+        g.phibar = g.sn * g.phibar;
+        g.pending = 1;
+        if (g.phibar <= a.tol * g.beta1 || g.beta == 0.0) g.active = 0;
+      }
+      sc[lane] = g;
+    }
+    __syncthreads();
+    double *const yo = r1;
+    r1 = r2;
+    r2 = y;
+    y = yo;
+    double *const wo = w2;
+    w2 = w;
+    w = wo;
   }
-  double b2;
-  if (!tile_reduce(sum, a.k, a.part, a.counters, b2)) return;
-  if (warp != 0 || !act) return;
-  m.oldb = m.beta;
-  m.beta = sqrt(b2);
-  m.oldeps = m.epsln;
-  m.delta = m.cs * m.dbar + m.sn * m.alfa;
-  const double gbar = m.sn * m.dbar - m.cs * m.alfa;
-  m.epsln = m.sn * m.beta;
-  m.dbar = -m.cs * m.beta;
-  double gam = sqrt(gbar * gbar + m.beta * m.beta);
-  if (!(gam > 1e-300)) gam = 1e-300;
-  m.gamma = gam;
-  m.cs = gbar / gam;
-  m.sn = m.beta / gam;
-  m.phi = m.cs * m.phibar;
-  m.phibar = m.sn * m.phibar;
-  m.pending = 1;
-  if (m.phibar <= a.tol * m.beta1 || m.beta == 0.0) m.active = 0;
-  a.s[c] = m;
+  if (warp == 0 && blockIdx.x == 0 && cl < a.k) a.s[cl] = sc[lane];
 }
 __global__ void minres_count_kernel(int k, const MinresScal *s, int *count) {
   int c = 0;
@@ -473,13 +522,21 @@ struct AdjBuffers {
   int *flag;
 };
 
-// Row blocks of the column sums: 16 rows at least, at most 4 blocks a SM and tile.
-static int adj_rows(int64_t n) {
-  const int64_t most = 4 * (int64_t)device_sm_count();
-  const int64_t r = std::max<int64_t>(16, (n + most - 1) / most);
+// Row blocks of the column sums and of the MINRES loop (all resident at once): 16 rows at least.
+static int adj_rows(int64_t n, int blocks) {
+  const int64_t r = std::max<int64_t>(16, (n + blocks - 1) / blocks);
   return (int)((r + kAdjWarps - 1) / kAdjWarps * kAdjWarps);
 }
-size_t adj_part_doubles(int k) { return 4 * (size_t)device_sm_count() * k; }
+// Resident blocks of the loop per tile of 32 columns.
+static int minres_blocks(int k) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, minres_loop_kernel, 32 * kAdjWarps, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return std::min(per_sm, 4) * device_sm_count() / ((k + 31) / 32);
+}
+size_t adj_part_doubles(int k) { return 2 * 4 * (size_t)device_sm_count() * k; }
 size_t adj_scal_bytes(int k) { return ((size_t)k * sizeof(MinresScal) + 255) / 256 * 256; }
 
 // The caller (slrf.cu) provides n x k scratch blocks (X here has leading dimension k).
@@ -489,7 +546,9 @@ int eig_grad_vectors(int64_t n, const int64_t *rowptr, const int32_t *col, const
                      cudaStream_t st) {
   const int64_t tot = n * k;
   const unsigned gb = (unsigned)((tot + 255) / 256);
-  const int rows = adj_rows(n);
+  const int blocks = minres_blocks(k);
+  if (blocks < 1) return SLRF_ECUDA;
+  const int rows = adj_rows(n, blocks);
   const dim3 grid((unsigned)((n + rows - 1) / rows), (unsigned)((k + 31) / 32));
   const int cw = k <= 8 ? 8 : (k <= 16 ? 16 : 32);
   auto colprod = [&](const double *x, const double *y, double *out) {
@@ -505,37 +564,46 @@ int eig_grad_vectors(int64_t n, const int64_t *rowptr, const int32_t *col, const
   cudaMemsetAsync(bf.w, 0, tot * sizeof(double), st);
   cudaMemsetAsync(bf.w2, 0, tot * sizeof(double), st);
   MinresArgs a{n, k, rows, rowptr, col, valA, valB, evals, bf.r, bf.b, bf.y, bf.w, bf.w2, bf.x, bf.scal, bf.part,
-               bf.counters, tol};
-  // the buffers after a step: r1 = r2, r2 = y, and the w just written in front
-  auto rotate = [&] {
-    double *const w = a.w2;
-    a.w2 = const_cast<double *>(a.w);
-    a.w = w;
-    double *const y = const_cast<double *>(a.r1);
-    a.r1 = a.r2;
-    a.r2 = a.y;
-    a.y = y;
+               bf.counters, bf.flag, tol, 0, cw};
+  cudaMemsetAsync(bf.flag, 0, 2 * sizeof(int), st);
+  // one launch of `steps` steps; the barrier counters start and end at zero
+  auto run = [&](int steps) {
+    a.steps = steps;
+    void *args[] = {&a};
+    cudaMemsetAsync(bf.counters, 0, grid.y * sizeof(unsigned), st);
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel((void *)minres_loop_kernel, grid, dim3(32 * kAdjWarps), args, 0, st);
+    cudaMemsetAsync(bf.counters, 0, grid.y * sizeof(unsigned), st);
+    for (int j = 0; j < steps; ++j) {  // the buffers after a step: r1 = r2, r2 = y, w2 in front
+      double *const y = a.r1;
+      a.r1 = a.r2;
+      a.r2 = a.y;
+      a.y = y;
+      std::swap(a.w, a.w2);
+    }
+    return e == cudaSuccess;
   };
   *notconv = 0;
   *h_active = 0;
   int itn = 0;
   while (itn < maxit) {
     const int chunk = maxit - itn < 64 ? maxit - itn : 64;
-    for (int j = 0; j < chunk; ++j) {
-      ++itn;
-      minres_apply_kernel<true><<<grid, 32 * kAdjWarps, 0, st>>>(a, cw);
-      minres_update_kernel<<<grid, 32 * kAdjWarps, 0, st>>>(a);
-      rotate();
-    }
+    itn += chunk;
+    if (!run(chunk)) return SLRF_ECUDA;
     // how many columns still iterate: stop early when none
     minres_count_kernel<<<1, 128, 0, st>>>(k, bf.scal, bf.flag + 1);
-    if (cudaMemcpyAsync(h_active, bf.flag + 1, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    int h[2] = {0, 0};
+    if (cudaMemcpyAsync(h_active, bf.flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return SLRF_ECUDA;
+    h[0] = h_active[0];
+    h[1] = h_active[1];
+    *h_active = h[1];
+    if (h[0] != 0) return SLRF_ETIMEOUT;  // a bounded barrier gave up
     if (*h_active == 0) break;
   }
   if (maxit > 0 && itn >= maxit && *h_active > 0) *notconv = 1;
-  minres_apply_kernel<false><<<grid, 32 * kAdjWarps, 0, st>>>(a, cw);  // pending w and x updates
+  if (!run(0)) return SLRF_ECUDA;  // pending w and x updates
   // B-orthogonal projection, then the pattern gradients
   spmm_real(n, rowptr, col, valA, valB, bf.x, k, k, nullptr, bf.BV, k, st);
   colprod(X, bf.BV, bf.work);  // x^T B xi
