@@ -233,7 +233,7 @@ struct MinresScal {
 // rotate through three buffers (no copies), v = r2 / beta is never stored (A v = (A r2) / beta),
 // and the w and x update of a step, which needs only the row's own entries, rides on the next
 // step's apply.  n = 2,002, k = 16: 11 launches a step and column sums of 512 rows on a thread
-// 240 us, two launches a step 26 us, now 16 us (two barriers, the latency of the gathers and
+// 240 us, two launches a step 26 us, now 15 us (two barriers, the latency of the gathers and
 // of the FP64 roots).
 constexpr int kAdjWarps = 8;
 

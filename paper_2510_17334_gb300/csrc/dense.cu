@@ -961,20 +961,27 @@ void chol_inv(int k, double *G, int ldg, double *Rinv, int ldr, int *status, cud
 // ------------------------------------------------------------------------------ Jacobi
 // Two-sided cyclic Jacobi with the round-robin (circle) ordering, which makes the kk/2
 // rotations of one round disjoint.  One block per pair: every block computes all rotations
-// of the round (cheap 2x2 problems), then rewrites the rows p, q of J^T A J and of V^T for
-// its own pair; one grid barrier per round.  The rotation inputs of a round (a_pp, a_qq,
-// a_pq of every pair) are not read from A, whose rows the owning blocks rewrite during the
-// round, but from a small table that the owners of the previous round filled (two copies,
-// alternating by round), and the block's own rows load together with them: a round costs
-// one L2 round trip, the rotation arithmetic and the barrier.  The sweep loop stops once
-// every off-diagonal met in a sweep is below 1e-9 of its diagonal scale (quadratic
-// convergence leaves them at rounding level after that sweep; at 1e-8 the clusters of a cube's
-// spectrum were left at up to 5e-9 of it).
+// of the round (cheap 2x2 problems), then rewrites the rows p, q of J^T A J for its own pair;
+// one grid barrier per round.  V^T takes rotations of its rows only, so each block keeps two of
+// its columns in shared memory and rotates them between its arrival at the barrier and the
+// wait.  The rotation inputs of a round (a_pp, a_qq, a_pq of every pair) are not read from A,
+// whose rows the owning blocks rewrite during the round, but from a small table that the owners
+// of the previous round filled (two copies, alternating by round), and the block's own rows
+// load together with them: a round costs one L2 round trip, the rotation arithmetic and the
+// barrier (k = 160: 3.37 -> 2.87 ms since V^T left the rows and the barrier is a release).  The
+// sweep loop stops once every off-diagonal met in a sweep is below 1e-9 of its diagonal scale
+// (quadratic convergence leaves them at rounding level after that sweep; at 1e-8 the clusters
+// of a cube's spectrum were left at up to 5e-9 of it).
 __device__ __forceinline__ void rr_pair(int kk, int r, int b, int &p, int &q) {
   const int M = kk - 1;
   int a0, a1;
   if (b == 0) { a0 = r; a1 = kk - 1; }
-  else { a0 = (r + b) % M; a1 = (r - b + M) % M; }
+  else {  // r + b and r - b modulo M (0 <= r < M, 0 < b < M)
+    a0 = r + b;
+    if (a0 >= M) a0 -= M;
+    a1 = r - b;
+    if (a1 < 0) a1 += M;
+  }
   p = a0 < a1 ? a0 : a1;
   q = a0 < a1 ? a1 : a0;
 }
@@ -982,7 +989,10 @@ __device__ __forceinline__ int rr_partner(int kk, int r, int x) {
   const int M = kk - 1;
   if (x == kk - 1) return r;
   if (x == r) return kk - 1;
-  return ((2 * r - x) % M + M) % M;
+  int y = 2 * r - x;  // modulo M; in (-M, 2M)
+  if (y < 0) y += M;
+  else if (y >= M) y -= M;
+  return y;
 }
 
 // Rotation (c, s) that annihilates a_pq: t = tan(phi) is the smaller root of
@@ -1031,23 +1041,27 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
   const unsigned nb = gridDim.x;  // == kk / 2: block b owns pair b of every round
   GridBarrier gb{w.bar, w.err};
   unsigned epoch = 0;
-  double *A = w.A, *Vt = w.Vt;
+  double *A = w.A;
   double *const rdiag = w.rot, *const roff = w.rot + 2 * kk;  // [2][kk] each
-  // init: A = H (padded), Vt = I
+  __shared__ double rp[512], rq[512];  // rows p, q of A
+  __shared__ double cs[512][2];        // rotation (c, s) of every index for this round
+  __shared__ double vt[2][512];        // columns 2 blockIdx.x and the next one of V^T
+  const int b0 = blockIdx.x;
+  // init: A = H (padded), V^T = I
+  for (int t = threadIdx.x; t < kk; t += blockDim.x) {
+    vt[0][t] = t == 2 * b0 ? 1.0 : 0.0;
+    vt[1][t] = t == 2 * b0 + 1 ? 1.0 : 0.0;
+  }
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)kk * kk;
        t += (int64_t)nb * blockDim.x) {
     const int i = (int)(t / kk), j = (int)(t % kk);
     const double h = (i < k && j < k) ? H[(size_t)i * ldh + j] : 0.0;
     A[t] = h;
-    Vt[t] = (i == j) ? 1.0 : 0.0;
     // the round-0 table: diagonal, and a_pq of every round-0 pair (p < q) at index p
     if (i == j) rdiag[i] = h;
     else if (i < j && rr_partner(kk, 0, i) == j) roff[i] = h;
   }
   if (!grid_sync(gb, nb, epoch)) return;
-  __shared__ double rp[512], rq[512];  // rows p, q of A
-  __shared__ double cs[512][2];        // rotation (c, s) of every index for this round
-  const int b0 = blockIdx.x;
   int par = 0;  // table copy of the current round
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     // has this thread met |a_pq| >= 2^-30 sqrt(|a_pp a_qq|) this sweep?  (identical in every
@@ -1056,16 +1070,14 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
     for (int r = 0; r < kk - 1; ++r) {
       int p, q;
       rr_pair(kk, r, b0, p, q);
-      // this block's rows of A and V^T, in flight while the rotation inputs load
-      double ap[kJacobiPer], aq[kJacobiPer], vp[kJacobiPer], vq[kJacobiPer];
+      // this block's rows of A, in flight while the rotation inputs load
+      double ap[kJacobiPer], aq[kJacobiPer];
 #pragma unroll
       for (int u = 0; u < kJacobiPer; ++u) {
         const int x = threadIdx.x + u * kJacobiThreads;
         if (x < kk) {
           ap[u] = __ldcg(&A[(size_t)p * kk + x]);
           aq[u] = __ldcg(&A[(size_t)q * kk + x]);
-          vp[u] = __ldcg(&Vt[(size_t)p * kk + x]);
-          vq[u] = __ldcg(&Vt[(size_t)q * kk + x]);
         }
       }
       // every block computes every rotation of the round (kk/2 independent 2x2 problems),
@@ -1108,8 +1120,6 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
           const double np = c * ajp - sn * ajq, nq = sn * ajp + c * ajq;
           A[(size_t)p * kk + x] = np;
           A[(size_t)q * kk + x] = nq;
-          Vt[(size_t)p * kk + x] = c * vp[u] - sn * vq[u];
-          Vt[(size_t)q * kk + x] = sn * vp[u] + c * vq[u];
           if (x == p) rdiag[nxt * kk + p] = np;
           if (x == q) rdiag[nxt * kk + q] = nq;
           if (x == pn && p < pn) roff[nxt * kk + p] = np;
@@ -1117,28 +1127,34 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
         }
       }
       par = nxt;
-      if (!grid_sync(gb, nb, epoch)) return;
+      grid_arrive(gb);
+      for (int t = threadIdx.x; t < kk; t += blockDim.x) {  // pair t / 2, column t & 1
+        int pb, qb;
+        rr_pair(kk, r, t >> 1, pb, qb);
+        double *const v = vt[t & 1];
+        const double cb = cs[pb][0], sb = cs[pb][1], vp = v[pb], vq = v[qb];
+        v[pb] = cb * vp - sb * vq;
+        v[qb] = sb * vp + cb * vq;
+      }
+      if (!grid_wait(gb, nb, epoch)) return;
     }
     if (!__syncthreads_or(unconv)) break;
   }
-  // sort ascending (stable by index) and write theta, S (column i = eigenvector i)
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-      const double di = __ldcg(&A[(size_t)i * kk + i]);
-      int rank = 0;
-      for (int j = 0; j < k; ++j) {
-        const double dj = __ldcg(&A[(size_t)j * kk + j]);
-        rank += (dj < di) || (dj == di && j < i);
-      }
-      theta[rank] = di;
-      for (int x = 0; x < k; ++x) S[(size_t)x * lds + rank] = __ldcg(&Vt[(size_t)i * kk + x]);
+  // sort ascending (stable by index) and write theta, S (column i = eigenvector i); the last
+  // round's table holds the diagonal, and a block has two rows of S
+  double *const d = rp;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) d[i] = __ldcg(&rdiag[par * kk + i]);
+  __syncthreads();
+  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    const double di = d[i];
+    int rank = 0;
+    for (int j = 0; j < k; ++j) {
+      const double dj = d[j];
+      rank += (dj < di) || (dj == di && j < i);
     }
+    if (b0 == 0) theta[rank] = di;
+    for (int x = 2 * b0; x < 2 * b0 + 2 && x < k; ++x) S[(size_t)x * lds + rank] = vt[x & 1][i];
   }
-}
-
-size_t jacobi_work_doubles(int k) {
-  const int kk = k + (k & 1);
-  return 2 * (size_t)kk * kk + 4 * (size_t)kk;
 }
 
 int jacobi_eig(int k, const double *H, int ldh, double *theta, double *S, int lds, JacobiWork w, cudaStream_t st) {

@@ -59,13 +59,11 @@ void chol_inv(int k, double *G, int ldg, double *Rinv, int ldr, int *status, cud
 // theta ascending (k), S (k x k row-major, column i = eigenvector i).
 struct JacobiWork {
   double *A;        // kk x kk
-  double *Vt;       // kk x kk
   double *rot;      // 4 * kk: diagonal and pair entries of the next round, two copies
   int *flags;       // [4]
   unsigned *bar;    // [2] barrier counters
   int *err;         // [1]
 };
-size_t jacobi_work_doubles(int k);
 int jacobi_eig(int k, const double *H, int ldh, double *theta, double *S, int lds, JacobiWork w,
                cudaStream_t st);
 
