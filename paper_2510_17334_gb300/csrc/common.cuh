@@ -90,14 +90,18 @@ template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 
 // Last-block handshake: every block calls this after writing its partials; exactly one
 // block (the last to arrive) gets true, and then sees all partials written before.
-// The caller resets *counter to 0 when the last block is done.
+// The caller resets *counter to 0 when the last block is done.  One acquire-release add orders
+// the stores and loads of the whole block (through the barriers around it); a full fence in every
+// thread cost 0.9 us of each launch (78 launches of 31 x 30 nodes, 12 columns: 1.28 -> 1.21 ms).
 __device__ __forceinline__ bool last_block_arrive(unsigned *counter, unsigned total) {
   __shared__ bool am_last;
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) am_last = (atomicAdd(counter, 1u) == total - 1u);
+  if (threadIdx.x == 0) {
+    unsigned seen;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(seen) : "l"(counter) : "memory");
+    am_last = seen == total - 1u;
+  }
   __syncthreads();
-  if (am_last) __threadfence();
   return am_last;
 }
 
