@@ -92,8 +92,9 @@ typedef struct {
   int group;              /* rows per group of the COCG SpMM's grouped-row format (rows of a
                              group share one union column list, so each gathered row feeds
                              all of them): 0 = choose (timed when autotune = 1, else from a
-                             cost model of the pattern), 1 = plain CSR, 2..4 = that many;
-                             default 0 */
+                             cost model of the pattern; a mixed-precision scalar pencil on a box
+                             keeps plain rows and goes through bricks, 32 rows that stage their
+                             gathered rows once), 1 = plain CSR, 2..4 = that many; default 0 */
   int bdiag;              /* 1 = with 3-row groups, use B-diagonal records when the pattern
                              allows: a vector-valued pencil whose B couples a dof only with the
                              same dof of a neighbour node (B = M (x) I_3, node-major dofs) keeps
