@@ -432,9 +432,10 @@ __global__ void __launch_bounds__(32 * kAdjWarps) minres_loop_kernel(const Minre
       }
     }
     if (!more) {
-      __syncthreads();
+      // a block may get here before another one has read a.s: the scalars are written back below,
+      // behind a barrier
+      if (!grid_sync(gb, gridDim.x, epoch)) return;
       if (warp == 0) sc[lane].pending = 0;
-      __syncthreads();
       break;
     }
     block_part(own && ok ? sum : 0.0, partA, a.k, sm);
@@ -490,7 +491,8 @@ __global__ void __launch_bounds__(32 * kAdjWarps) minres_loop_kernel(const Minre
     w2 = w;
     w = wo;
   }
-  if (warp == 0 && blockIdx.x == 0 && cl < a.k) a.s[cl] = sc[lane];
+  // epoch 0: nothing was done and no barrier passed since the blocks read a.s
+  if (epoch > 0 && warp == 0 && blockIdx.x == 0 && cl < a.k) a.s[cl] = sc[lane];
 }
 __global__ void minres_count_kernel(int k, const MinresScal *s, int *count) {
   int c = 0;
