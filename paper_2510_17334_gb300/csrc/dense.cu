@@ -731,8 +731,10 @@ constexpr size_t kCholSmemMax = 220 * 1024;
 //   chol_panel_kernel: every CTA factors the diagonal block D = G[j0.., j0..] itself (a
 //     32 x 32 problem in shared memory), then the rows [j1 + 32 blockIdx.x, +32) of the
 //     panel below: L[i][j0 + c] = (G[i][j0 + c] - sum_{l < c} L[i][j0 + l] D[c][l]) / D[c][c];
+//     with more than one CTA the factor of D goes to R^{-1}'s storage, which is free until
+//     tri_inv_kernel, since a CTA may start when CTA 0 has finished already;
 //   chol_syrk_kernel: the trailing lower triangle G[i][l] -= sum_c L[i][j0 + c] L[l][j0 + c],
-//     one CTA per 32 x 32 tile (i >= l);
+//     one CTA per 32 x 32 tile (i >= l); CTA 0 moves the factor of D into G;
 //   tri_inv_kernel: X = L^{-1} by blocks of kCi columns (one CTA each), rows in blocks of kCi:
 //     X[I][C] = L[I][I]^{-1} (E[I][C] - L[I][<I] X[<I][C]), stored as R^{-1}[c][i] = X[i][c].
 // A pivot that is not positive (or not finite) raises *status (SLRF_ECHOL); every kernel
@@ -746,8 +748,8 @@ constexpr int kCholBlockedMin = SLRF_CHOL_BLOCKED_MIN;  // smallest k for the bl
 __device__ __forceinline__ bool chol_skip(const int *status, const int *run_if) {
   return (run_if != nullptr && *run_if == 0) || *reinterpret_cast<const volatile int *>(status) != 0;
 }
-__global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int ldg, int j0, int *status,
-                                                         const int *run_if) {
+__global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int ldg, int j0, double *F, int ldf,
+                                                         int *status, const int *run_if) {
   if (chol_skip(status, run_if)) return;
   __shared__ double D[kCb][kCb + 1];
   __shared__ int fail;
@@ -789,7 +791,7 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int l
   if (blockIdx.x == 0)
     for (int e = tid; e < b * b; e += blockDim.x) {
       const int i = e / b, l = e % b;
-      if (l <= i) G[(size_t)(j0 + i) * ldg + j0 + l] = D[i][l];
+      if (l <= i) F[(size_t)(j0 + i) * ldf + j0 + l] = D[i][l];
     }
   // panel rows of this CTA: forward substitution with D^T, column by column; thread (row, part)
   // of the first four warps keeps the columns part, part + 4, ...
@@ -831,9 +833,14 @@ __global__ void __launch_bounds__(256) chol_panel_kernel(int k, double *G, int l
     if (rr < nr && c < b) G[(size_t)(r0 + rr) * ldg + j0 + c] = P[rr][c];
   }
 }
-__global__ void __launch_bounds__(256) chol_syrk_kernel(int k, double *G, int ldg, int j0, int b, int *status,
-                                                        const int *run_if) {
+__global__ void __launch_bounds__(256) chol_syrk_kernel(int k, double *G, int ldg, int j0, int b, const double *F,
+                                                        int ldf, int *status, const int *run_if) {
   if (chol_skip(status, run_if)) return;
+  if (blockIdx.x == 0 && F != G)
+    for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
+      const int i = e / b, l = e % b;
+      if (l <= i) G[(size_t)(j0 + i) * ldg + j0 + l] = F[(size_t)(j0 + i) * ldf + j0 + l];
+    }
   // tile (ti, tj), ti >= tj, from the linear block index
   int t = (int)blockIdx.x, ti = 0;
   while (t > ti) { t -= ti + 1; ++ti; }
@@ -924,10 +931,12 @@ static void chol_inv_blocked(int k, double *G, int ldg, double *Rinv, int ldr, i
     const int b = std::min(kCb, k - j0);
     const int rest = k - j0 - b;
     const int pb = std::max(1, (rest + kCb - 1) / kCb);
-    chol_panel_kernel<<<pb, 256, 0, st>>>(k, G, ldg, j0, status, run_if);
+    double *const F = pb > 1 ? Rinv : G;
+    const int ldf = pb > 1 ? ldr : ldg;
+    chol_panel_kernel<<<pb, 256, 0, st>>>(k, G, ldg, j0, F, ldf, status, run_if);
     if (rest > 0) {
       const int T = (rest + 31) / 32;
-      chol_syrk_kernel<<<T * (T + 1) / 2, 256, 0, st>>>(k, G, ldg, j0, b, status, run_if);
+      chol_syrk_kernel<<<T * (T + 1) / 2, 256, 0, st>>>(k, G, ldg, j0, b, F, ldf, status, run_if);
     }
   }
   const size_t smem = (size_t)k * kCi * sizeof(double);
