@@ -1030,6 +1030,11 @@ __device__ __forceinline__ void jacobi_rotation(double app, double aqq, double a
     return;
   }
   const float tf = scale_f(th, 1023 - em), pf = scale_f(ph, 1023 - em);
+  if (pf == 0.f) {  // a_pq below 2^-149 of th, or both subnormal (0 / 0 below)
+    c = 1.0;
+    sn = 0.0;
+    return;
+  }
   const float at = fabsf(tf);
   float t = __fdividef(pf, at + sqrtf(fmaf(tf, tf, pf * pf)));
   t = tf > 0.f ? t : (tf < 0.f ? -t : fabsf(t));  // th = 0: t = 1
@@ -1099,9 +1104,10 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(int k, int kk, c
         // a_pq^2 against a_pp a_qq by exponents alone (within a factor of 4, no FP64 operation)
         const int gap = exp_bits(app) + exp_bits(aqq) - 2 * exp_bits(apq);
         const bool nz = (__double_as_longlong(apq) & 0x7FFFFFFFFFFFFFFFll) != 0;
-        unconv |= nz && gap <= 60;
         double c = 1.0, sn = 0.0;
         if (nz && gap < 100) jacobi_rotation(app, aqq, apq, c, sn);
+        // a pair that was left alone (not finite, subnormal) is no reason for another sweep
+        unconv |= gap <= 60 && __double_as_longlong(sn) != 0;
         cs[pb][0] = c; cs[pb][1] = sn;
         cs[qb][0] = c; cs[qb][1] = sn;
       }
