@@ -1845,9 +1845,7 @@ template <typename R, int G> static void grp_attrs() {
                            grp_smem_bytes<float, 3, true>());
   }
 }
-void cocg_kernel_attrs() {
-  static bool done = false;
-  if (done) return;
+static void set_kernel_attrs() {
   constexpr int sm64 = grp_smem_bytes<double, 3, true>();
   cudaFuncSetAttribute(spmm_grp_real64_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
   cudaFuncSetAttribute(spmm_grp_real64_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
@@ -1864,7 +1862,10 @@ void cocg_kernel_attrs() {
   cudaFuncSetAttribute(cocg_brick_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
   cudaFuncSetAttribute(cocg_brick_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmemMax);
   cudaGetLastError();
-  done = true;
+}
+void cocg_kernel_attrs() {
+  static OncePerDevice once;
+  once(set_kernel_attrs);
 }
 template <typename R, int G, bool BD> static int grp_occ() {
   int b = 0;

@@ -220,4 +220,19 @@ inline int device_sm_count() {
   return v;
 }
 
+// Function attributes (shared memory beyond 48 KB) belong to the device that is current: a kernel's
+// are set once on each device that it runs on.  f may run again, for instance in two threads at
+// once.
+struct OncePerDevice {
+  static constexpr int kMaxDev = 64;
+  std::atomic<bool> done[kMaxDev] = {};
+  template <typename F> void operator()(F &&f) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) dev = 0;
+    if (dev < kMaxDev && done[dev].load(std::memory_order_acquire)) return;
+    f();
+    if (dev < kMaxDev) done[dev].store(true, std::memory_order_release);
+  }
+};
+
 }  // namespace slrf

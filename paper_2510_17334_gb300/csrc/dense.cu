@@ -945,21 +945,16 @@ static void chol_inv_blocked(int k, double *G, int ldg, double *Rinv, int ldr, i
 
 void chol_inv(int k, double *G, int ldg, double *Rinv, int ldr, int *status, cudaStream_t st, const int *run_if,
               bool fp32) {
-  static bool attrs = false;
-  if (!attrs) {
+  static OncePerDevice once;
+  once([] {
     cudaFuncSetAttribute(chol_inv_smem_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemMax);
     cudaFuncSetAttribute(chol_inv_smem_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemMax);
-    attrs = true;
-  }
+    cudaFuncSetAttribute(tri_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemMax);
+  });
   const size_t b64 = ((size_t)k * k + 3 * k) * sizeof(double), b32 = ((size_t)k * k + 3 * k) * sizeof(float);
-  if (k >= kCholBlockedMin && (size_t)k * kCi * sizeof(double) <= kCholSmemMax) {
-    static bool tri_attr = false;
-    if (!tri_attr) {
-      cudaFuncSetAttribute(tri_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemMax);
-      tri_attr = true;
-    }
+  if (k >= kCholBlockedMin && (size_t)k * kCi * sizeof(double) <= kCholSmemMax)
     chol_inv_blocked(k, G, ldg, Rinv, ldr, status, st, run_if);
-  } else if (fp32 && b32 <= kCholSmemMax)
+  else if (fp32 && b32 <= kCholSmemMax)
     chol_inv_smem_kernel<float><<<1, 1024, b32, st>>>(k, G, ldg, Rinv, ldr, status, run_if);
   else if (b64 <= kCholSmemMax)
     chol_inv_smem_kernel<double><<<1, 1024, b64, st>>>(k, G, ldg, Rinv, ldr, status, run_if);

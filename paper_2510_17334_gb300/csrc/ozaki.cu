@@ -514,11 +514,11 @@ __global__ void oz_gram_finalize_kernel(int k1, int k2, int nsplit, int MR, int 
 int num_sms() { return device_sm_count(); }
 
 void set_smem_attrs() {
-  static bool done = false;
-  if (done) return;
-  cudaFuncSetAttribute(oz_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaSmem);
-  cudaFuncSetAttribute(oz_split_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kS * 64 * 8 * 16);
-  done = true;
+  static OncePerDevice once;
+  once([] {
+    cudaFuncSetAttribute(oz_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaSmem);
+    cudaFuncSetAttribute(oz_split_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kS * 64 * 8 * 16);
+  });
 }
 
 struct GramPlan {
