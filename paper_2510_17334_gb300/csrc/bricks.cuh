@@ -217,7 +217,8 @@ __global__ void brick_count_kernel(int64_t ngroups, const int64_t *__restrict__ 
 // the CSR rows, the brick's row list is their sorted union, and every record gets its values and
 // the place of its row in the list.  *flag is raised where a brick has more rows than kBrickRows,
 // a pair more columns than cmax, a row is not sorted, or a pair's own rows are not among its
-// columns; stats: staged rows, records, rows of the largest brick.
+// columns; stats: staged rows, records, rows of the largest brick.  Without rec only these are
+// found.
 constexpr int kBrickSort = 2048;  // >= kBrickGroups * cmax (checked by the host)
 __global__ void __launch_bounds__(256) brick_build_kernel(const int64_t *__restrict__ rowptr,
                                                           const int32_t *__restrict__ col,
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(256) brick_build_kernel(const int64_t *__restr
     if (tid == 0) atomicExch(flag, 1);
     return;
   }
-  if (tid < kBrickGroups) {
+  if (rec != nullptr && tid < kBrickGroups) {
     groups[(size_t)b * kBrickGroups + tid] = g;
     unsigned char *const base = rec + ((size_t)b * kBrickGroups + tid) * gs;
     float4 *const val = reinterpret_cast<float4 *>(base);

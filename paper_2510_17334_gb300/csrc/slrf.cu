@@ -97,7 +97,7 @@ struct slrf_ctx {
   Bricks bricks{};                   // mixed path: staged SpMM format (count 0: not in use)
   bool batched = false;              // a problem of a batch: lane width 2 in FP32
   unsigned char *grec64 = nullptr;   // mixed path: FP64 B-diagonal records of the same groups
-  double *x64 = nullptr;             // padded FP64 copy of a real block for the grouped FP64 products
+  double *x64 = nullptr;             // row-scaled FP64 copy of a real block for the grouped FP64 products
   // real n x L blocks (ld = L)
   double *V = nullptr, *AV = nullptr, *BV = nullptr, *G = nullptr, *AG = nullptr, *BG = nullptr;
   double *U = nullptr, *U2 = nullptr, *BU = nullptr, *Vt = nullptr, *AVt = nullptr, *BVt = nullptr;
@@ -120,6 +120,7 @@ struct slrf_ctx {
   int it_cur = 0;  // It_max of the next filter apply (opts.it_adapt: grows per problem)
   int unres_streak = 0;  // consecutive outer steps with the lowest active Ritz pair unresolved
   std::vector<void *> allocs;
+  size_t reserve = 0;  // group = 0: bytes that the rest of the setup will allocate (see dalloc_spare)
 };
 
 // ----------------------------------------------------------------------------- helpers
@@ -151,6 +152,15 @@ template <typename T> static int dalloc(slrf_ctx *ctx, T **p, size_t count) {
   ctx->allocs.push_back(q);
   *p = reinterpret_cast<T *>(q);
   return SLRF_OK;
+}
+
+// Memory of an SpMM format that the setup may do without: SLRF_ENOMEM unless the rest of the working
+// set still fits beside it.
+template <typename T> static int dalloc_spare(slrf_ctx *ctx, T **p, size_t count) {
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return SLRF_ECUDA;
+  if (count * sizeof(T) + ctx->reserve > fr) return SLRF_ENOMEM;
+  return dalloc(ctx, p, count);
 }
 
 static void dfree(slrf_ctx *ctx, void *p) {
@@ -280,6 +290,14 @@ static void drop_groups(slrf_ctx *ctx) {
 static int build_groups(slrf_ctx *ctx, int G) {
   drop_groups(ctx);
   if (G <= 1) return SLRF_OK;
+  unsigned char *bdrec = nullptr, *gen64 = nullptr, *bd64 = nullptr;
+  auto give_up = [&](int rc) {
+    dfree(ctx, bdrec);
+    dfree(ctx, gen64);
+    dfree(ctx, bd64);
+    drop_groups(ctx);
+    return rc;
+  };
   std::vector<int> cnt;
   int rc = group_counts(ctx, G, cnt);
   if (rc != SLRF_OK) return rc;
@@ -287,8 +305,9 @@ static int build_groups(slrf_ctx *ctx, int G) {
   std::vector<int64_t> off((size_t)ng + 1, 0);
   for (int64_t g = 0; g < ng; ++g) off[g + 1] = off[g] + cnt[g];
   // gptr[ng + 1] (one spare word) holds the record check's flag
-  if ((rc = dalloc(ctx, &ctx->gptr, (size_t)ng + 2)) != SLRF_OK) return rc;
-  if ((rc = dalloc(ctx, &ctx->grec, (size_t)grec_span_rt(off[ng], G, ctx->mixed) + 16)) != SLRF_OK) return rc;
+  if ((rc = dalloc_spare(ctx, &ctx->gptr, (size_t)ng + 2)) != SLRF_OK) return give_up(rc);
+  if ((rc = dalloc_spare(ctx, &ctx->grec, (size_t)grec_span_rt(off[ng], G, ctx->mixed) + 16)) != SLRF_OK)
+    return give_up(rc);
   if (cudaMemcpyAsync(ctx->gptr, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, ctx->st) !=
       cudaSuccess)
     return SLRF_ECUDA;
@@ -324,8 +343,8 @@ static int build_groups(slrf_ctx *ctx, int G) {
         cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
       return SLRF_ECUDA;
     if (nbd == 0) {
-      unsigned char *bdrec = nullptr;
-      if ((rc = dalloc(ctx, &bdrec, (size_t)grec_span_rt(off[ng], 3, ctx->mixed, true) + 16)) != SLRF_OK) return rc;
+      if ((rc = dalloc_spare(ctx, &bdrec, (size_t)grec_span_rt(off[ng], 3, ctx->mixed, true) + 16)) != SLRF_OK)
+        return give_up(rc);
       if (ctx->mixed) grp_bd_convert<float>(off[ng], ctx->grec, bdrec, ctx->st);
       else grp_bd_convert<double>(off[ng], ctx->grec, bdrec, ctx->st);
       if (cudaMemsetAsync(dflag, 0, sizeof(int), ctx->st) != cudaSuccess) return SLRF_ECUDA;
@@ -334,19 +353,16 @@ static int build_groups(slrf_ctx *ctx, int G) {
       if (cudaMemcpyAsync(&bad, dflag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st) != cudaSuccess ||
           cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
         return SLRF_ECUDA;
-      if (bad) {
-        dfree(ctx, bdrec);
-        drop_groups(ctx);
-        return SLRF_EINVAL;
-      }
+      if (bad) return give_up(SLRF_EINVAL);
       dfree(ctx, ctx->grec);
       ctx->grec = bdrec;
+      bdrec = nullptr;
       bd = 1;
       if (ctx->mixed) {
         // FP64 B-diagonal records of the same groups for the FP64 real products of the outer step
-        unsigned char *gen64 = nullptr, *bd64 = nullptr;
-        if ((rc = dalloc(ctx, &gen64, (size_t)grec_span_rt(off[ng], 3, false) + 16)) != SLRF_OK) return rc;
-        if ((rc = dalloc(ctx, &bd64, (size_t)grec_span_rt(off[ng], 3, false, true) + 16)) != SLRF_OK) return rc;
+        if ((rc = dalloc_spare(ctx, &gen64, (size_t)grec_span_rt(off[ng], 3, false) + 16)) != SLRF_OK ||
+            (rc = dalloc_spare(ctx, &bd64, (size_t)grec_span_rt(off[ng], 3, false, true) + 16)) != SLRF_OK)
+          return give_up(rc);
         grp_fill<double>(ctx->n, 3, ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), ctx->gptr, gen64, ctx->st);
         grp_bd_convert<double>(off[ng], gen64, bd64, ctx->st);
         if (cudaMemsetAsync(dflag, 0, sizeof(int), ctx->st) != cudaSuccess) return SLRF_ECUDA;
@@ -355,8 +371,10 @@ static int build_groups(slrf_ctx *ctx, int G) {
             cudaStreamSynchronize(ctx->st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
           return SLRF_ECUDA;
         dfree(ctx, gen64);
+        gen64 = nullptr;
         if (bad) dfree(ctx, bd64);
         else ctx->grec64 = bd64;
+        bd64 = nullptr;
       }
     }
   }
@@ -422,7 +440,8 @@ static void mesh_strides(const std::vector<int32_t> &cols, int64_t row, int64_t 
 // 4 x 4 x 2 rows (8 x 4 in a plane, 32 in a line).  Kept where the bricks stage at most 0.6 rows
 // per record they multiply (27-point pattern 0.25, 9-point 0.3, a line 0.53); without locality in
 // the numbering, or with rows too long for the shared memory of two blocks, the grouped or CSR
-// kernel stays.
+// kernel stays.  So it does (SLRF_ENOMEM, bricks.count 0) when the bricks do not fit beside the
+// rest of the working set; the records are allocated once the bricks are known to pay.
 static int build_bricks(slrf_ctx *ctx) {
   drop_bricks(ctx);
   if (!ctx->mixed) return SLRF_OK;
@@ -479,13 +498,13 @@ static int build_bricks(slrf_ctx *ctx) {
   unsigned char *rec = nullptr;
   unsigned long long *stats = nullptr;  // staged rows, records, largest brick, longest group, flag
   int rc;
-  if ((rc = dalloc(ctx, &dg, groups.size())) != SLRF_OK) return rc;
+  if ((rc = dalloc_spare(ctx, &dg, groups.size())) != SLRF_OK) return rc;
   B.groups = dg;
-  if ((rc = dalloc(ctx, &dn, (size_t)B.count)) != SLRF_OK) return give_up(rc);
+  if ((rc = dalloc_spare(ctx, &dn, (size_t)B.count)) != SLRF_OK) return give_up(rc);
   B.nrows = dn;
-  if ((rc = dalloc(ctx, &dr, (size_t)B.count * kBrickRows)) != SLRF_OK) return give_up(rc);
+  if ((rc = dalloc_spare(ctx, &dr, (size_t)B.count * kBrickRows)) != SLRF_OK) return give_up(rc);
   B.rows = dr;
-  if ((rc = dalloc(ctx, &stats, 5)) != SLRF_OK) return give_up(rc);
+  if ((rc = dalloc_spare(ctx, &stats, 5)) != SLRF_OK) return give_up(rc);
   unsigned long long h[5] = {};
   cudaMemsetAsync(stats, 0, 5 * sizeof(unsigned long long), ctx->st);
   cudaMemcpyAsync(dg, groups.data(), groups.size() * sizeof(int4), cudaMemcpyHostToDevice, ctx->st);
@@ -497,14 +516,17 @@ static int build_bricks(slrf_ctx *ctx) {
   }
   const int cmax = (int)h[3];
   bool fit = cmax >= 1 && kBrickGroups * cmax <= 2048;
-  if (fit) {
+  for (int pass = 0; fit && pass < 2; ++pass) {  // the staged rows, then the records too
     B.group_bytes = brick_group_size(cmax, B.pad);
-    rc = dalloc(ctx, &rec, (size_t)B.count * kBrickGroups * B.group_bytes);
-    if (rc != SLRF_OK) {
-      dfree(ctx, stats);
-      return give_up(rc);
+    if (pass == 1) {
+      rc = dalloc_spare(ctx, &rec, (size_t)B.count * kBrickGroups * B.group_bytes);
+      if (rc != SLRF_OK) {
+        dfree(ctx, stats);
+        return give_up(rc);
+      }
+      B.rec = rec;
     }
-    B.rec = rec;
+    cudaMemsetAsync(stats, 0, 5 * sizeof(unsigned long long), ctx->st);
     brick_build(ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), B.count, cmax, B.pad, B.group_bytes, dg, dn,
                 dr, rec, reinterpret_cast<int *>(stats + 4), stats, ctx->st);
     cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, ctx->st);
@@ -521,12 +543,16 @@ static int build_bricks(slrf_ctx *ctx) {
   return SLRF_OK;
 }
 
-// Bricks for the COCG SpMM if the pattern has them, with pairs of rows (records) for the real
-// products; otherwise the groups stay as they are.
+// Bricks for the COCG SpMM if the pattern has them and they fit, with pairs of rows (records) for
+// the real products; otherwise the groups stay as they are (plain rows, if the pairs do not fit).
 static int use_bricks(slrf_ctx *ctx) {
   int rc = build_bricks(ctx);
-  if (rc != SLRF_OK || ctx->bricks.count == 0) return rc;
-  if (ctx->grp != 2 && (rc = build_groups(ctx, 2)) != SLRF_OK) return rc;
+  if (rc != SLRF_OK && rc != SLRF_ENOMEM) return rc;
+  if (ctx->bricks.count == 0) return SLRF_OK;
+  if (ctx->grp != 2 && (rc = build_groups(ctx, 2)) != SLRF_OK) {
+    drop_bricks(ctx);
+    return rc == SLRF_ENOMEM ? SLRF_OK : rc;
+  }
   ctx->vec = cocg_vec_csr<float>();  // 64-entry tiles
   return SLRF_OK;
 }
@@ -535,10 +561,12 @@ static int setup_groups(slrf_ctx *ctx) {
   int G = ctx->o.group;
   if (G == 0) {
     int rc = choose_group(ctx, G);
-    if (rc != SLRF_OK) return rc;
+    if (rc == SLRF_ENOMEM) G = 1;
+    else if (rc != SLRF_OK) return rc;
   }
+  // a height that was not asked for gives way to plain rows when its records do not fit
   int rc = build_groups(ctx, G);
-  if (rc != SLRF_OK) return rc;
+  if (rc != SLRF_OK && !(rc == SLRF_ENOMEM && ctx->o.group == 0)) return rc;
   // bricks before groups of any height, but for vector-valued pencils (B-diagonal records)
   if (ctx->o.group == 0 && !ctx->bdiag && (rc = use_bricks(ctx)) != SLRF_OK) return rc;
   // the batched kernels run bricks or plain CSR, at the CSR lane width
@@ -902,7 +930,9 @@ static int autotune_rows(slrf_ctx *ctx) {
     for (int g = 1; g <= 4; ++g) {
       if (g > 1 && !ctx->mixed && g != g_model) continue;
       drop_bricks(ctx);
-      if ((rc = build_groups(ctx, g)) != SLRF_OK) break;
+      rc = build_groups(ctx, g);
+      if (rc == SLRF_ENOMEM) { rc = SLRF_OK; continue; }
+      if (rc != SLRF_OK) break;
       ctx->rpb_tuned = 0;
       if ((rc = time_spmm(t)) != SLRF_OK) break;
       if (t < best) { best = t; best_g = g; best_bricks = false; }
@@ -1459,6 +1489,11 @@ static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int
     to_float_kernel<<<gb, 256, 0, ctx->st>>>(ctx->nnz, cocg_valA(ctx), ctx->valA32);
     to_float_kernel<<<gb, 256, 0, ctx->st>>>(ctx->nnz, cocg_valB(ctx), ctx->valB32);
   }
+  const size_t ozbytes = o.dense ? oz_work_bytes(n, L, L) : 0;
+  // gram() splits rows into at most 64 chunks of k1 x k2 <= L x L partial tiles
+  ctx->work_doubles = std::max({(size_t)64 * L * L, ritz_work_doubles(n, L), (size_t)4 * L});
+  if (o.group == 0)
+    ctx->reserve = need - matrix + ozbytes + 8 * (ctx->work_doubles + 8 * (size_t)L * L + (size_t)n) + (64u << 20);
   if ((rc = setup_groups(ctx)) != SLRF_OK) return fail(rc);
   AL(ctx->iflags, 16);
   if (cudaMallocHost(&ctx->h_iflags, 16 * sizeof(int)) != cudaSuccess) return fail(SLRF_ENOMEM);
@@ -1532,11 +1567,9 @@ static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int
   AL(ctx->theta, L); AL(ctx->theta_act, L); AL(ctx->res, L); AL(ctx->res_paper, L); AL(ctx->sgn, L);
   AL(ctx->Theta, L); AL(ctx->Res, L);
   AL(ctx->dst_x, L); AL(ctx->dst_v, L);
-  // gram() splits rows into at most 64 chunks of k1 x k2 <= L x L partial tiles
-  ctx->work_doubles = std::max({(size_t)64 * L * L, ritz_work_doubles(n, L), (size_t)4 * L});
   AL(ctx->work, ctx->work_doubles);
   if (o.dense) {
-    ctx->ozwork_bytes = oz_work_bytes(n, L, L);
+    ctx->ozwork_bytes = ozbytes;
     AL(ctx->ozwork, ctx->ozwork_bytes);
   }
   {
@@ -1548,6 +1581,7 @@ static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int
     ctx->jw.err = ctx->iflags + 9;
   }
 #undef AL
+  ctx->reserve = 0;
   for (auto &e : ctx->ev)
     if (cudaEventCreate(&e) != cudaSuccess) return fail(SLRF_ECUDA);
   if (o.autotune) {
