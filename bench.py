@@ -481,14 +481,14 @@ def main():
     # kernel-level roofline of the dominant kernel (the fused shifted SpMM + COCG phase 1)
     with torch.cuda.stream(stream):
         tim = ctx.filter_timing(V0[:, :wl.block])
-    fmt = ctx.format()
+    fmt, bricks = ctx.format(), ctx.bricks()[0]
     ctx.close()
     spmm_ms = tim["ms_spmm"] / max(tim["n_spmm"], 1)
     traffic = args.traffic_bytes
     if traffic is None and args.group == 0:
         traffic = DEFAULT_TRAFFIC.get((args.workload, prec))
     roof = spmm_roofline(p, wl.m, wl.block, prec, spmm_ms, traffic, bdiag=fmt[1] == 1)
-    roof["spmm_format"] = {"group": fmt[0], "b_diagonal": fmt[1], "lane_width": fmt[2]}
+    roof["spmm_format"] = {"group": fmt[0], "b_diagonal": fmt[1], "lane_width": fmt[2], "bricks": bricks}
     roof["update_ms"] = tim["ms_update"] / max(tim["n_update"], 1)
     roof["spmm_ms"] = spmm_ms
     # ---- the other precision on the same workload (FP64 vs mixed at equal residual)

@@ -92,9 +92,9 @@ typedef struct {
   int group;              /* rows per group of the COCG SpMM's grouped-row format (rows of a
                              group share one union column list, so each gathered row feeds
                              all of them): 0 = choose (timed when autotune = 1, else from a
-                             cost model of the pattern; a mixed-precision scalar pencil on a box
-                             keeps plain rows and goes through bricks, 32 rows that stage their
-                             gathered rows once), 1 = plain CSR, 2..4 = that many; default 0 */
+                             cost model of the pattern; a mixed-precision scalar pencil whose
+                             numbering has the locality of a box goes through bricks, pairs of
+                             rows gathered into 32 that stage their gathered rows once), 1 = plain CSR, 2..4 = that many; default 0 */
   int bdiag;              /* 1 = with 3-row groups, use B-diagonal records when the pattern
                              allows: a vector-valued pencil whose B couples a dof only with the
                              same dof of a neighbour node (B = M (x) I_3, node-major dofs) keeps
@@ -335,11 +335,18 @@ void slrf_destroy(slrf_ctx *ctx);
 const char *slrf_strerror(int status);
 
 /* The COCG SpMM format the context chose at setup (host outputs, any may be NULL): *group =
- * rows per group (1 = plain CSR), *bdiag = 1 when the grouped records are B-diagonal (see
+ * rows that share one list of columns (1 = plain CSR; 2 with bricks, whose records are of row
+ * pairs, see slrf_bricks), *bdiag = 1 when the grouped records are B-diagonal (see
  * slrf_opts.bdiag), *lane_width = complex entries per lane of the COCG kernels (FP64 1, FP32 2
  * or 4).  The paper has no counterpart; it reports the data layout of Sec. 4's inner solves.
  * Errors: SLRF_EINVAL (NULL ctx). */
 int slrf_format(const slrf_ctx *ctx, int *group, int *bdiag, int *lane_width);
+
+/* Bricks of the COCG SpMM (host outputs, any may be NULL): *count = bricks of at most 32 rows that
+ * stage their gathered rows once in shared memory (0 = the format of slrf_format without bricks),
+ * *staged_rows = rows that the largest of them stages.  The paper has no counterpart.
+ * Errors: SLRF_EINVAL (NULL ctx). */
+int slrf_bricks(const slrf_ctx *ctx, int *count, int *staged_rows);
 
 /* First error recorded in the context (SLRF_OK if none). */
 int slrf_last_error(const slrf_ctx *ctx);

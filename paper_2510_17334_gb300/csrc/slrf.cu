@@ -1624,6 +1624,13 @@ int slrf_format(const slrf_ctx *ctx, int *group, int *bdiag, int *lane_width) {
   return SLRF_OK;
 }
 
+int slrf_bricks(const slrf_ctx *ctx, int *count, int *staged_rows) {
+  if (!ctx) return SLRF_EINVAL;
+  if (count) *count = ctx->bricks.count;
+  if (staged_rows) *staged_rows = ctx->bricks.count > 0 ? ctx->bricks.max_rows : 0;
+  return SLRF_OK;
+}
+
 int slrf_apply(slrf_ctx *ctx, const double *X, int k, double *AX, double *BX, int fp32) {
   if (!ctx) return SLRF_EINVAL;
   if (ctx->status != SLRF_OK) return SLRF_ESTATE;

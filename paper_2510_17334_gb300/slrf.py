@@ -33,7 +33,7 @@ SYMBOLS = ("slrf_opts_default", "slrf_setup", "slrf_get_poles", "slrf_filter_app
            "slrf_rayleigh_ritz", "slrf_solve", "slrf_solve_host", "slrf_eig_grad", "slrf_destroy",
            "slrf_strerror", "slrf_last_error", "slrf_filter_apply_static", "slrf_setup_batched",
            "slrf_solve_batched", "slrf_destroy_batched", "slrf_tsgram", "slrf_tsgemm", "slrf_wait_selftest",
-           "slrf_apply", "slrf_format")
+           "slrf_apply", "slrf_format", "slrf_bricks")
 
 
 class SlrfError(RuntimeError):
@@ -83,6 +83,7 @@ def lib() -> ct.CDLL:
         L.slrf_filter_apply.argtypes = [vp, vp, i, vp, vp]
         L.slrf_apply.argtypes = [vp, vp, i, vp, vp, i]
         L.slrf_format.argtypes = [vp, ct.POINTER(i), ct.POINTER(i), ct.POINTER(i)]
+        L.slrf_bricks.argtypes = [vp, ct.POINTER(i), ct.POINTER(i)]
         L.slrf_filter_stats.argtypes = [vp, vp, vp, vp]
         L.slrf_filter_timing.argtypes = [vp, vp, i, vp, vp, vp, vp]
         L.slrf_rayleigh_ritz.argtypes = [vp, vp, i, vp, vp, i, i, vp, vp, vp]
@@ -200,6 +201,12 @@ class Context:
         g, bd, lw = ct.c_int(), ct.c_int(), ct.c_int()
         _check(lib().slrf_format(self.h, ct.byref(g), ct.byref(bd), ct.byref(lw)), "slrf_format")
         return g.value, bd.value, lw.value
+
+    def bricks(self):
+        """(count, staged_rows) of the COCG SpMM's bricks, (0, 0) without them (see slrf_bricks)."""
+        c, r = ct.c_int(), ct.c_int()
+        _check(lib().slrf_bricks(self.h, ct.byref(c), ct.byref(r)), "slrf_bricks")
+        return c.value, r.value
 
     def apply(self, X: torch.Tensor, fp32: bool = False, want_a: bool = True, want_b: bool = True):
         """(A X, B X) with the context's matrices (see slrf_apply); an output not wanted is None."""
