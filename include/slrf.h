@@ -348,6 +348,9 @@ int slrf_format(const slrf_ctx *ctx, int *group, int *bdiag, int *lane_width);
  * Errors: SLRF_EINVAL (NULL ctx). */
 int slrf_bricks(const slrf_ctx *ctx, int *count, int *staged_rows);
 
+/* The same for problem p (0 <= p < P) of a batch; the other problems have no say in it. */
+int slrf_batch_bricks(const slrf_batch *batch, int p, int *count, int *staged_rows);
+
 /* First error recorded in the context (SLRF_OK if none). */
 int slrf_last_error(const slrf_ctx *ctx);
 

@@ -33,7 +33,8 @@ SYMBOLS = ("slrf_opts_default", "slrf_setup", "slrf_get_poles", "slrf_filter_app
            "slrf_rayleigh_ritz", "slrf_solve", "slrf_solve_host", "slrf_eig_grad", "slrf_destroy",
            "slrf_strerror", "slrf_last_error", "slrf_filter_apply_static", "slrf_setup_batched",
            "slrf_solve_batched", "slrf_destroy_batched", "slrf_tsgram", "slrf_tsgemm", "slrf_wait_selftest",
-           "slrf_apply", "slrf_format", "slrf_bricks")
+           "slrf_apply", "slrf_format", "slrf_bricks",
+           "slrf_batch_bricks")
 
 
 class SlrfError(RuntimeError):
@@ -84,6 +85,7 @@ def lib() -> ct.CDLL:
         L.slrf_apply.argtypes = [vp, vp, i, vp, vp, i]
         L.slrf_format.argtypes = [vp, ct.POINTER(i), ct.POINTER(i), ct.POINTER(i)]
         L.slrf_bricks.argtypes = [vp, ct.POINTER(i), ct.POINTER(i)]
+        L.slrf_batch_bricks.argtypes = [vp, i, ct.POINTER(i), ct.POINTER(i)]
         L.slrf_filter_stats.argtypes = [vp, vp, vp, vp]
         L.slrf_filter_timing.argtypes = [vp, vp, i, vp, vp, vp, vp]
         L.slrf_rayleigh_ritz.argtypes = [vp, vp, i, vp, vp, i, i, vp, vp, vp]
@@ -313,6 +315,12 @@ class Batch:
             self.close()
         except Exception:
             pass
+
+    def bricks(self, p: int):
+        """(count, staged_rows) of problem p (see slrf_batch_bricks)."""
+        c, r = ct.c_int(), ct.c_int()
+        _check(lib().slrf_batch_bricks(self.h, p, ct.byref(c), ct.byref(r)), "slrf_batch_bricks")
+        return c.value, r.value
 
     def solve(self, V0=None, caps=None, check=True):
         caps = np.ascontiguousarray(self.blocks if caps is None else caps, dtype=np.int32)
