@@ -1955,7 +1955,7 @@ int slrf_setup_batched(slrf_batch **out, int P, const slrf_csr_pair *pencils, co
   slrf_opts ob;
   if (opts) ob = *opts;
   else slrf_opts_default(&ob);
-  ob.group = ob.precision == 1 ? 0 : 1;
+  ob.group = ob.precision == 1 && ob.group == 0 ? 0 : 1;  // other heights have no batched kernel
   for (int p = 0; p < P; ++p) {
     const int rc = setup_impl(&b->c[p], &pencils[p], gammas[p], blocks[p], &ob, stream, true);
     if (rc != SLRF_OK) {

@@ -39,3 +39,10 @@ def test_batches_of_both_formats(slrf_mod, names, opts):  # noqa: F811
         assert status == 0 and nf == 8
         assert np.all(np.abs(ev.cpu().numpy() - lam[:8]) <= 1e-8 * lam[:8])
     b.close()
+
+
+def test_a_batch_honours_plain_rows(slrf_mod):  # noqa: F811
+    """slrf_opts.group = 1 asks for plain CSR in a batch as in a single context."""
+    b, _, _ = _batch(slrf_mod, ["box", "plane"], group=1)
+    assert b.bricks(0) == b.bricks(1) == (0, 0)
+    b.close()
