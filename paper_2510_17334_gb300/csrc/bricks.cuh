@@ -203,6 +203,27 @@ __device__ __forceinline__ int brick_place(const int *list, int n, int m) {
   }
   return lo;
 }
+// Key of the longest row, the one next to row n / 2 of several (the lower one of two): its length,
+// then 2^31 - 1 less the distance, then whether it is not above.  One atomic per block.
+__global__ void __launch_bounds__(256) longest_row_kernel(int64_t n, const int64_t *__restrict__ rowptr,
+                                                          unsigned long long *key) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long k = 0;
+  if (i < n) {
+    const int64_t len = rowptr[i + 1] - rowptr[i], d = i - n / 2;
+    k = ((unsigned long long)(len < 0xFFFFFFFF ? len : 0xFFFFFFFF) << 32) |
+        (unsigned long long)((0x7FFFFFFF - (d < 0 ? -d : d)) << 1 | (d <= 0));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, o));
+  __shared__ unsigned long long w[8];
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = k;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) k = max(k, w[q]);
+    atomicMax(key, k);
+  }
+}
 // Most records of a pair.
 __global__ void brick_count_kernel(int64_t ngroups, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
                                    const double *__restrict__ valA, const double *__restrict__ valB,

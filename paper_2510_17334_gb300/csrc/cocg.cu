@@ -1622,6 +1622,14 @@ int brick_group_size(int cmax, int &pad) {
   pad = brick_pad(cmax);
   return brick_group_bytes(cmax);
 }
+void longest_row(int64_t n, const int64_t *rowptr, unsigned long long *key, cudaStream_t st) {
+  longest_row_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, rowptr, key);
+}
+void longest_row_of(unsigned long long key, int64_t n, int64_t &len, int64_t &row) {
+  len = (int64_t)(key >> 32);
+  const int64_t d = 0x7FFFFFFF - (int64_t)((key & 0xFFFFFFFFull) >> 1);
+  row = (key & 1) ? n / 2 - d : n / 2 + d;
+}
 void brick_count(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int64_t ngroups,
                  const int4 *groups, unsigned long long *most, cudaStream_t st) {
   brick_count_kernel<<<(unsigned)((ngroups + 127) / 128), 128, 0, st>>>(ngroups, rowptr, col, valA, valB, groups, most);

@@ -265,6 +265,10 @@ void spmm_grp_real64(int64_t n, int64_t ngroups, const int64_t *gptr, const unsi
 // Brick format: bytes of a group's record area, and the build (see bricks.cuh; groups holds
 // (first row, rows) on entry).
 int brick_group_size(int cmax, int &pad);
+// Longest row of the pattern (of several the one next to the middle) as a key, from zero, and what
+// the key says.
+void longest_row(int64_t n, const int64_t *rowptr, unsigned long long *key, cudaStream_t st);
+void longest_row_of(unsigned long long key, int64_t n, int64_t &len, int64_t &row);
 void brick_count(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int64_t ngroups,
                  const int4 *groups, unsigned long long *most, cudaStream_t st);
 void brick_build(const int64_t *rowptr, const int32_t *col, const double *valA, const double *valB, int count, int cmax,

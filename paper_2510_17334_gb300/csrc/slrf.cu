@@ -120,6 +120,7 @@ struct slrf_ctx {
   int it_cur = 0;  // It_max of the next filter apply (opts.it_adapt: grows per problem)
   int unres_streak = 0;  // consecutive outer steps with the lowest active Ritz pair unresolved
   std::vector<void *> allocs;
+  std::vector<int> gcnt[5];  // union sizes of the heights looked at (setup_groups)
   size_t reserve = 0;  // group = 0: bytes that the rest of the setup will allocate (see dalloc_spare)
 };
 
@@ -251,18 +252,23 @@ __global__ void final_gather_kernel(int64_t n, int nconv, int cnt, const int *ra
 
 // ----------------------------------------------------------------------------- grouped rows
 // The COCG SpMM's grouped-row format (CocgArgs): rows [G g, G g + G) share one union
-// column list.  group_counts returns the union sizes for a G; build_groups writes the
+// column list.  group_counts finds the union sizes for a few heights; build_groups writes the
 // offsets and the records of the working precision; choose_group picks G.
-static int group_counts(slrf_ctx *ctx, int G, std::vector<int> &cnt) {
-  const int64_t ng = (ctx->n + G - 1) / G;
+static int group_counts(slrf_ctx *ctx, std::initializer_list<int> heights) {
   int *d = nullptr;
-  if (cudaMalloc(&d, (size_t)ng * sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(&d, (size_t)(ctx->n + 1) * sizeof(int)) != cudaSuccess) {  // enough for every height
     cudaGetLastError();
     return SLRF_ENOMEM;
   }
-  grp_count(ctx->n, G, ctx->rowptr, ctx->col, d, ctx->st);
-  cnt.resize((size_t)ng);
-  cudaError_t e = cudaMemcpyAsync(cnt.data(), d, (size_t)ng * sizeof(int), cudaMemcpyDeviceToHost, ctx->st);
+  cudaError_t e = cudaSuccess;
+  for (int G : heights) {
+    const int64_t ng = (ctx->n + G - 1) / G;
+    std::vector<int> &cnt = ctx->gcnt[G];
+    cnt.resize((size_t)ng);
+    grp_count(ctx->n, G, ctx->rowptr, ctx->col, d, ctx->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(cnt.data(), d, (size_t)ng * sizeof(int), cudaMemcpyDeviceToHost, ctx->st);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->st);
   cudaFree(d);
   return e == cudaSuccess ? SLRF_OK : SLRF_ECUDA;
@@ -298,9 +304,10 @@ static int build_groups(slrf_ctx *ctx, int G) {
     drop_groups(ctx);
     return rc;
   };
-  std::vector<int> cnt;
-  int rc = group_counts(ctx, G, cnt);
-  if (rc != SLRF_OK) return rc;
+  int rc = SLRF_OK;
+  if (ctx->gcnt[G].empty() && (rc = group_counts(ctx, {G})) != SLRF_OK) return rc;
+  const std::vector<int> cnt = std::move(ctx->gcnt[G]);
+  ctx->gcnt[G].clear();
   const int64_t ng = (int64_t)cnt.size();
   std::vector<int64_t> off((size_t)ng + 1, 0);
   for (int64_t g = 0; g < ng; ++g) off[g + 1] = off[g] + cnt[g];
@@ -358,7 +365,7 @@ static int build_groups(slrf_ctx *ctx, int G) {
       ctx->grec = bdrec;
       bdrec = nullptr;
       bd = 1;
-      if (ctx->mixed) {
+      if (ctx->mixed && !ctx->batched) {
         // FP64 B-diagonal records of the same groups for the FP64 real products of the outer step
         if ((rc = dalloc_spare(ctx, &gen64, (size_t)grec_span_rt(off[ng], 3, false) + 16)) != SLRF_OK ||
             (rc = dalloc_spare(ctx, &bd64, (size_t)grec_span_rt(off[ng], 3, false, true) + 16)) != SLRF_OK)
@@ -394,10 +401,10 @@ static int build_groups(slrf_ctx *ctx, int G) {
 static int choose_group(slrf_ctx *ctx, int &G) {
   G = 1;
   double best = (double)ctx->nnz / ctx->n;
+  const int rc = group_counts(ctx, {2, 3, 4});
+  if (rc != SLRF_OK) return rc;
   for (int g = (ctx->mixed ? 2 : 4); ctx->mixed ? g <= 4 : g >= 2; g += ctx->mixed ? 1 : -1) {
-    std::vector<int> cnt;
-    int rc = group_counts(ctx, g, cnt);
-    if (rc != SLRF_OK) return rc;
+    const std::vector<int> &cnt = ctx->gcnt[g];
     double recs = 0, slots = 0;
     for (size_t i = 0; i < cnt.size(); ++i) {
       recs += cnt[i];
@@ -441,28 +448,30 @@ static void mesh_strides(const std::vector<int32_t> &cols, int64_t row, int64_t 
 // per record they multiply (27-point pattern 0.25, 9-point 0.3, a line 0.53); without locality in
 // the numbering, or with rows too long for the shared memory of two blocks, the grouped or CSR
 // kernel stays.  So it does (SLRF_ENOMEM, bricks.count 0) when the bricks do not fit beside the
-// rest of the working set; the records are allocated once the bricks are known to pay.
+// rest of the working set.  A record area larger than the CSR values (nearly empty bricks: lines or
+// planes of two rows) is allocated only when a first pass has shown that the bricks pay.
 static int build_bricks(slrf_ctx *ctx) {
   drop_bricks(ctx);
   if (!ctx->mixed) return SLRF_OK;
   const int64_t n = ctx->n;
-  std::vector<int64_t> rp((size_t)n + 1);
-  if (cudaMemcpyAsync(rp.data(), ctx->rowptr, rp.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->st) !=
-          cudaSuccess ||
+  // the longest row, the one next to the middle of several
+  unsigned long long *key = nullptr, hkey = 0;
+  int rc = dalloc_spare(ctx, &key, 1);
+  if (rc != SLRF_OK) return rc;
+  cudaMemsetAsync(key, 0, sizeof(*key), ctx->st);
+  longest_row(n, ctx->rowptr, key, ctx->st);
+  const bool ok = cudaMemcpyAsync(&hkey, key, sizeof(hkey), cudaMemcpyDeviceToHost, ctx->st) == cudaSuccess &&
+                  cudaStreamSynchronize(ctx->st) == cudaSuccess;
+  dfree(ctx, key);
+  if (!ok) return SLRF_ECUDA;
+  int64_t longest, row, rs = 0;
+  longest_row_of(hkey, n, longest, row);
+  if (longest < 1 || longest > 128) return SLRF_OK;
+  if (cudaMemcpyAsync(&rs, ctx->rowptr + row, sizeof(rs), cudaMemcpyDeviceToHost, ctx->st) != cudaSuccess ||
       cudaStreamSynchronize(ctx->st) != cudaSuccess)
     return SLRF_ECUDA;
-  // the longest row, the one next to the middle of several
-  int64_t row = n / 2, longest = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    const int64_t len = rp[i + 1] - rp[i];
-    if (len > longest || (len == longest && std::llabs(i - n / 2) < std::llabs(row - n / 2))) {
-      longest = len;
-      row = i;
-    }
-  }
-  if (longest < 1 || longest > 128) return SLRF_OK;
   std::vector<int32_t> cols((size_t)longest);
-  if (cudaMemcpyAsync(cols.data(), ctx->col + rp[row], cols.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
+  if (cudaMemcpyAsync(cols.data(), ctx->col + rs, cols.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
                       ctx->st) != cudaSuccess ||
       cudaStreamSynchronize(ctx->st) != cudaSuccess)
     return SLRF_ECUDA;
@@ -497,7 +506,6 @@ static int build_bricks(slrf_ctx *ctx) {
   int *dn = nullptr, *dr = nullptr;
   unsigned char *rec = nullptr;
   unsigned long long *stats = nullptr;  // staged rows, records, largest brick, longest group, flag
-  int rc;
   if ((rc = dalloc_spare(ctx, &dg, groups.size())) != SLRF_OK) return rc;
   B.groups = dg;
   if ((rc = dalloc_spare(ctx, &dn, (size_t)B.count)) != SLRF_OK) return give_up(rc);
@@ -516,8 +524,9 @@ static int build_bricks(slrf_ctx *ctx) {
   }
   const int cmax = (int)h[3];
   bool fit = cmax >= 1 && kBrickGroups * cmax <= 2048;
-  for (int pass = 0; fit && pass < 2; ++pass) {  // the staged rows, then the records too
-    B.group_bytes = brick_group_size(cmax, B.pad);
+  if (fit) B.group_bytes = brick_group_size(cmax, B.pad);
+  const bool small = (double)B.count * kBrickGroups * B.group_bytes <= 24.0 * ctx->nnz;
+  for (int pass = small ? 1 : 0; fit && pass < 2; ++pass) {  // the staged rows, then the records too
     if (pass == 1) {
       rc = dalloc_spare(ctx, &rec, (size_t)B.count * kBrickGroups * B.group_bytes);
       if (rc != SLRF_OK) {
@@ -558,18 +567,29 @@ static int use_bricks(slrf_ctx *ctx) {
 }
 
 static int setup_groups(slrf_ctx *ctx) {
-  int G = ctx->o.group;
-  if (G == 0) {
-    int rc = choose_group(ctx, G);
+  int G = ctx->o.group, rc;
+  const bool choose = G == 0;
+  struct Drop {  // the union sizes are of no use after this
+    slrf_ctx *c;
+    ~Drop() {
+      for (auto &v : c->gcnt) std::vector<int>().swap(v);
+    }
+  } drop{ctx};
+  if (choose) {
+    rc = choose_group(ctx, G);
     if (rc == SLRF_ENOMEM) G = 1;
     else if (rc != SLRF_OK) return rc;
   }
+  // bricks before groups of any height, but for vector-valued pencils (B-diagonal records, which only
+  // the 3-row groups themselves can show)
+  if (choose && G != 3) {
+    if ((rc = use_bricks(ctx)) != SLRF_OK || ctx->bricks.count > 0) return rc;
+    if (ctx->batched) return SLRF_OK;  // the batched kernels run bricks or plain CSR
+  }
   // a height that was not asked for gives way to plain rows when its records do not fit
-  int rc = build_groups(ctx, G);
-  if (rc != SLRF_OK && !(rc == SLRF_ENOMEM && ctx->o.group == 0)) return rc;
-  // bricks before groups of any height, but for vector-valued pencils (B-diagonal records)
-  if (ctx->o.group == 0 && !ctx->bdiag && (rc = use_bricks(ctx)) != SLRF_OK) return rc;
-  // the batched kernels run bricks or plain CSR, at the CSR lane width
+  rc = build_groups(ctx, G);
+  if (rc != SLRF_OK && !(rc == SLRF_ENOMEM && choose)) return rc;
+  if (choose && G == 3 && !ctx->bdiag && (rc = use_bricks(ctx)) != SLRF_OK) return rc;
   if (ctx->batched && ctx->bricks.count == 0) drop_groups(ctx);
   return SLRF_OK;
 }
