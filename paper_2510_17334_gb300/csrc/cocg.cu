@@ -1764,7 +1764,6 @@ struct GrpReal64 {
   int ldy;
   const double *yscale;
 };
-int grp_real64_ld(int k) { return (k + 63) / 64 * 64; }
 __global__ void to_f64_scaled_kernel(int64_t n, int k, const double *__restrict__ X, int ldx,
                                      const double *__restrict__ s, double *__restrict__ Y, int ldy) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

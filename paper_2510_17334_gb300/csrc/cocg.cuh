@@ -256,9 +256,8 @@ void grp_bd_detect(int64_t n, int64_t ngroups, const int64_t *gptr, const unsign
 template <typename R>
 void grp_bd_convert(int64_t nrec, const unsigned char *rec, unsigned char *bdrec, cudaStream_t st);
 // FP64 real products through FP64 B-diagonal records of 3-row groups: YA = A X and/or YB = B X
-// (either may be null), X first copied to x64 ([n][grp_real64_ld(k)], padding zero) with row i
-// multiplied by xscale[i] (null: 1), output row i by yscale[i] (null: 1).
-int grp_real64_ld(int k);
+// (either may be null), row i of X multiplied by xscale[i] in a copy, x64 (n x k; null: X itself, no
+// copy), output row i by yscale[i] (null: 1).
 void spmm_grp_real64(int64_t n, int64_t ngroups, const int64_t *gptr, const unsigned char *grec, int *err, int nrb,
                      const double *X, int ldx, int k, const double *xscale, double *x64, double *YA, double *YB,
                      int ldy, const double *yscale, cudaStream_t st);

@@ -97,7 +97,7 @@ struct slrf_ctx {
   Bricks bricks{};                   // mixed path: staged SpMM format (count 0: not in use)
   bool batched = false;              // a problem of a batch: lane width 2 in FP32
   unsigned char *grec64 = nullptr;   // mixed path: FP64 B-diagonal records of the same groups
-  double *x64 = nullptr;             // row-scaled FP64 copy of a real block for the grouped FP64 products
+  double *x64 = nullptr;             // precond: row-scaled FP64 copy of a real block (grouped FP64 products)
   // real n x L blocks (ld = L)
   double *V = nullptr, *AV = nullptr, *BV = nullptr, *G = nullptr, *AG = nullptr, *BG = nullptr;
   double *U = nullptr, *U2 = nullptr, *BU = nullptr, *Vt = nullptr, *AVt = nullptr, *BVt = nullptr;
@@ -632,7 +632,7 @@ static int grp_real_blocks(const slrf_ctx *ctx) {
 static void real_products64(slrf_ctx *ctx, const double *X, int ldx, int k, double *YA, double *YB, int ldy,
                             cudaStream_t st) {
   const unsigned char *r64 = rec64(ctx);
-  if (r64 != nullptr && ctx->x64 != nullptr)
+  if (r64 != nullptr)
     spmm_grp_real64(ctx->n, ctx->ngroups, ctx->gptr, r64, ctx->iflags + 15, grp_real_blocks(ctx), X, ldx, k,
                     ctx->dsqrt, ctx->x64, YA, YB, ldy, ctx->dsqrt, st);
   else
@@ -886,9 +886,9 @@ static int filter_prep(slrf_ctx *ctx, const double *X, int ldx, int k, const dou
                     ctx->G, L, k, nullptr, ctx->x32, ctx->AG, ctx->BG, L, nullptr, st, ctx->bdiag != 0);
   else if (ctx->mixed)
     spmm_ab32(ctx->n, ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), ctx->G, L, k, ctx->AG, ctx->BG, L, st);
-  else if (rec64(ctx) != nullptr && ctx->x64 != nullptr)  // records hold the values the solves use
+  else if (rec64(ctx) != nullptr)  // records hold the values the solves use
     spmm_grp_real64(ctx->n, ctx->ngroups, ctx->gptr, rec64(ctx), ctx->iflags + 15, grp_real_blocks(ctx), ctx->G, L, k,
-                    nullptr, ctx->x64, ctx->AG, ctx->BG, L, nullptr, st);
+                    nullptr, nullptr, ctx->AG, ctx->BG, L, nullptr, st);
   else
     spmm_real(ctx->n, ctx->rowptr, ctx->col, cocg_valA(ctx), cocg_valB(ctx), ctx->G, L, k, ctx->AG, ctx->BG, L, st);
   ctx->launches += 1;
@@ -1481,7 +1481,7 @@ static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int
   const size_t matrix = (size_t)ctx->nnz * (4 + 16 + (ctx->mixed ? 8 : 0)) + 8 * (size_t)(n + 1);
   const size_t refine = (ctx->mixed && o.refine_max > 1) ? 16 * (size_t)n * ctx->Wmax : 0;
   const size_t uacc = 8 * (size_t)n * (ctx->Wmax / ctx->mp) + (ctx->mixed ? 4 * (size_t)n * grp_real32_ld(L) : 0) +
-                      8 * (size_t)n * grp_real64_ld(L);
+                      (o.precond ? 8 * (size_t)n * L : 0);
   const size_t need = (state + blocks + matrix + refine + uacc) + 8 * partial + (64u << 20);
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return fail(SLRF_ECUDA);
@@ -1595,8 +1595,8 @@ static int setup_impl(slrf_ctx **out, const slrf_csr_pair *pc, double gamma, int
   }
   AL(ctx->uacc, (size_t)n * (ctx->Wmax / ctx->mp));
   if (ctx->mixed) AL(ctx->x32, (size_t)n * grp_real32_ld(L));
-  AL(ctx->x64, (size_t)n * grp_real64_ld(L));
   if (ctx->dsc != nullptr) {
+    AL(ctx->x64, (size_t)n * L);
     AL(ctx->dsqrt, (size_t)n);
     recip_kernel<<<(unsigned)((n + 255) / 256), 256, 0, ctx->st>>>(n, ctx->dsc, ctx->dsqrt);
   }

@@ -72,3 +72,20 @@ for dev in (0, 1, 3):
     assert lib.slrf_tsgram(n, u, k, k, u, k, k, v, k, 1, None) == 0, dev
     assert fake.fake_refused() == 0 and fake.fake_launches() > 20, dev
 """)
+
+
+def test_row_scaled_copy_only_with_the_preconditioner(run):
+    """The FP64 copy of a block with scaled rows (n x L doubles) is memory of preconditioned contexts
+    alone; beside it they hold four arrays of a row or an entry each."""
+    run("""
+n, k = 4096, 96
+p, keep = pencil(n)
+used = []
+for precond in (0, 1):
+    before = fake.fake_used()
+    rc, h = setup(p, k, precision=0, precond=precond)
+    assert rc == 0
+    used.append(fake.fake_used() - before)
+    lib.slrf_destroy(h)
+assert used[1] - used[0] >= 8 * n * k, used
+""")
