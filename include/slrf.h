@@ -228,7 +228,12 @@ int slrf_solve_host(const slrf_csr_pair *pencil_host, double gamma, int block_L,
  * in slrf_setup.  Each problem gets its own context and stream (its real sweeps and
  * Rayleigh-Ritz steps run concurrently); the COCG phases of all active problems run as
  * one persistent launch per phase over the work list of (problem, row block, column tile)
- * items, captured in a CUDA graph.  Errors: as slrf_setup (first failing problem). */
+ * items, captured in a CUDA graph.  A problem keeps the SpMM format it has by itself
+ * (slrf_opts.group = 0 and precision = 1: bricks, see slrf_batch_bricks, or plain CSR; otherwise
+ * plain CSR).  precision = 0: every result is bitwise that of a single solve with group = 1.
+ * precision = 1: the split of the rows follows all problems still active, so a problem's
+ * rounding depends on the others in the batch; a repeated solve gives the same bits.
+ * Errors: as slrf_setup (first failing problem). */
 int slrf_setup_batched(slrf_batch **batch, int P, const slrf_csr_pair *pencils, const double *gammas,
                        const int *blocks, const slrf_opts *opts, void *stream);
 
@@ -261,7 +266,8 @@ void slrf_destroy_batched(slrf_batch *batch);
  * NULL), outputs gA, gB (device nnz, overwritten).  The pattern is the context's; with
  * g_X the context's n x L work blocks are used as scratch (k <= L).
  * Errors: SLRF_EINVAL, SLRF_ENOCONV (some MINRES column missed its tolerance; the
- * gradients are still written), SLRF_ESTATE, SLRF_ECUDA. */
+ * gradients are still written), SLRF_ETIMEOUT (with g_X: a bounded device-side wait of the
+ * MINRES loop gave up; the context is then in its failed state), SLRF_ESTATE, SLRF_ECUDA. */
 int slrf_eig_grad(slrf_ctx *ctx, int k, const double *evals, const double *X, int ldx,
                   const double *g_eval, const double *g_X, double *gA, double *gB);
 

@@ -186,7 +186,8 @@ static int sddmm(int64_t n, const int64_t *rowptr, const int32_t *col, int k, co
                  const SdWeights &w, double *gA, double *gB, cudaStream_t st) {
   const size_t per_row = kSdWarps * (size_t)k * sizeof(double2);  // shared memory of one row per warp
   if (per_row > 200 * 1024) return SLRF_EINVAL;
-  // rows per warp: up to 8, within 56 KB a block (4 blocks of 8 warps a SM)
+  // rows per warp: up to 8, within 56 KB a block; with the 6.5 KB of queues and the 1 KB that the
+  // system keeps of each block three blocks of 8 warps share an SM (k = 50: 51,200 B)
   const int R = (int)std::max<size_t>(1, std::min<size_t>(8, (56 * 1024) / per_row));
   const size_t smem = per_row * R;
   const bool v2 = ldx % 2 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;

@@ -38,8 +38,8 @@ void shifted_residual(int64_t n, int k, const double *AV, const double *BV, int 
 // C (k1 x k2, row-major, ldc) = X^T Y for X (n x k1), Y (n x k2).  sym: X == Y, k1 == k2,
 // only upper tiles are computed and mirrored.  work must hold gram_work_doubles(...) doubles.
 size_t gram_work_doubles(int64_t n, int k1, int k2);
-// fp32: FP32 inputs and accumulation within row chunks (for passes whose error a later
-// FP64 pass removes); run_if: device flag, the launch does nothing while *run_if == 0.
+// f32 (n x (k1 + k2) floats, or null): FP32 copies of the inputs and accumulation within row chunks
+// (for passes whose error a later FP64 pass removes); run_if: device flag, the launch does nothing while *run_if == 0.
 void gram(int64_t n, const double *X, int ldx, int k1, const double *Y, int ldy, int k2, double *C, int ldc,
           bool sym, double *work, cudaStream_t st, float *f32 = nullptr, const int *run_if = nullptr);
 

@@ -445,11 +445,19 @@ static void mesh_strides(const std::vector<int32_t> &cols, int64_t row, int64_t 
 
 // Brick format of the FP32 SpMM (bricks.cuh): pairs of neighbouring rows gathered into bricks of
 // 4 x 4 x 2 rows (8 x 4 in a plane, 32 in a line).  Kept where the bricks stage at most 0.6 rows
-// per record they multiply (27-point pattern 0.25, 9-point 0.3, a line 0.53); without locality in
-// the numbering, or with rows too long for the shared memory of two blocks, the grouped or CSR
-// kernel stays.  So it does (SLRF_ENOMEM, bricks.count 0) when the bricks do not fit beside the
-// rest of the working set.  A record area larger than the CSR values (nearly empty bricks: lines or
-// planes of two rows) is allocated only when a first pass has shown that the bricks pay.
+// per record they multiply; without locality in the numbering, or with rows too long for the shared
+// memory of two blocks, the grouped or CSR kernel stays.  Staged rows per record, and a product of
+// 64 columns x 8 poles in microseconds on bricks / plain rows / pairs gathered through L1:
+//   27 points, 41^3 nodes            0.25      409 /   627 /  446
+//   9 points, 447^2                  0.3       836 / 1,299 /  891
+//   5 points, 447^2                  0.43      832 / 1,355 /  790
+//   7 points, 58^3                   0.48      836 / 1,363 /  898
+//   a line of 200,000                0.53      822 /   968 /  829
+// and with 8 columns the same ratios or better (a line 116 / 161 / 231).  A shuffled numbering
+// stages nearly a row per record.
+// The bricks also stay out (SLRF_ENOMEM, bricks.count 0) when they do not fit beside the rest of the
+// working set.  A record area larger than the CSR values (nearly empty bricks: lines or planes of
+// two rows) is allocated only when a first pass has shown that the bricks pay.
 static int build_bricks(slrf_ctx *ctx) {
   drop_bricks(ctx);
   if (!ctx->mixed) return SLRF_OK;
