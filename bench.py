@@ -45,10 +45,9 @@ DEFAULT_PRECOND = {"elast_32": 1, "elast_48": 1, "elast_64": 1}
 # DRAM bytes (read + write) of one full-width launch of the timed path's SpMM kernel, from
 # an ncu capture of the kernel as it is now (block 32, 2 tiles, scaled to the 30 tiles of
 # block 480; traffic is linear in the tiles), keyed by (workload, precision); an entry is
-# dropped when the kernel changes.  The grouped kernel with B-diagonal records read 74.2 GB
-# per launch when it staged 63 records a chunk; the node-triple records it stages now (27 a
-# chunk) have not been captured, so the roofline's traffic is null.
-DEFAULT_TRAFFIC = {}
+# dropped when the kernel changes.  Grouped kernel on node-triple records: 4.69 GB in 2 tiles
+# (74.2 GB per full launch with single-column records).
+DEFAULT_TRAFFIC = {("elast_64", 1): 70.4e9}
 
 
 def measured_hbm_gbs():

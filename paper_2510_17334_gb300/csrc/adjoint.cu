@@ -233,9 +233,9 @@ struct MinresScal {
 // block adds them itself in the same order, so nothing else is exchanged.  The Lanczos vectors
 // rotate through three buffers (no copies), v = r2 / beta is never stored (A v = (A r2) / beta),
 // and the w and x update of a step, which needs only the row's own entries, rides on the next
-// step's apply.  n = 2,002, k = 16: 11 launches a step and column sums of 512 rows on a thread
-// 240 us, two launches a step 26 us, now 15 us (two barriers, the latency of the gathers and
-// of the FP64 roots).
+// step's apply.  n = 2,002, k = 16, about 300 steps: the whole adjoint took 96.1 ms with 11 launches a
+// step and column sums of 512 rows on a thread, 9.9 ms with two launches a step, now 5.9 ms, 18 to
+// 19 us a step (two barriers, the latency of the gathers and of the FP64 roots).
 constexpr int kAdjWarps = 8;
 
 // Sum v over the warps of the block and then over the blocks of the tile (gridDim.x of them):
