@@ -8,7 +8,7 @@ n = 380,928, 29.6M stored entries, lognormal Young's modulus), gamma = 220.8176 
 eigenpairs below it), block 480, m = 8 poles, Jacobi-preconditioned inner solves, complex-FP32
 COCG in FP64 refinement (It_max 23); the same solve in FP64 is the "compare" record.  Other
 workloads (--workload): q1_lap_41 (3D Q1 Laplacian on 41^3 nodes), elast_32 / elast_48,
-bar1d_2000, batch64 (64 uneven pencils solved together), sens48 (48 scaled pencils).
+bar1d_2000, batch64 (64 uneven pencils solved together), sens48 (adjoint of a 48^3 elasticity box).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
